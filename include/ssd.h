@@ -210,7 +210,8 @@ int ssd_rewind(ssd_ctx* ctx, int32_t length);
 
 /* The skinny projection kernel alone: out[r][n] = sum_k x[r][k] * w[n][k] with bf16 operands and
  * fp32 accumulation, split over `split_k` K ranges that are summed in order.  DEVICE pointers:
- * x [rows, k] bf16, w [n, k] bf16, out [rows, n] fp32.  k a multiple of 8.  Test / tuning hook. */
+ * x [rows, k] bf16, w [n, k] bf16 (both on 16-byte boundaries), out [rows, n] fp32 (anywhere a float may
+ * lie).  k a multiple of 8.  Test / tuning hook. */
 int ssd_gemm_bf16(ssd_ctx* ctx, const void* x_dev, const void* w_dev, float* out_dev,
                   int32_t rows, int32_t n, int32_t k, int32_t split_k);
 
@@ -220,8 +221,9 @@ int ssd_gemm_bf16(ssd_ctx* ctx, const void* x_dev, const void* w_dev, float* out
  * device or run out of memory: neither can use a context, whose creation allocates.  This entry point
  * needs no context, calls no cudaMalloc/cudaFree nor any allocating library routine and uses no scratch
  * memory: a call is one kernel that sums its K splits on chip.
- *   x_dev [rows,k] bf16, w_dev [n,k] bf16, out_dev [rows,n] fp32: DEVICE memory of the current device,
- *   owned by the caller; k a multiple of 8; 1 <= split_k <= 8; `cuda_stream` a cudaStream_t.
+ *   x_dev [rows,k] bf16, w_dev [n,k] bf16 (both on 16-byte boundaries), out_dev [rows,n] fp32 (anywhere a float
+ *   may lie): DEVICE memory of the current device, owned by the caller; k a multiple of 8; 1 <= split_k <= 8;
+ *   `cuda_stream` a cudaStream_t.
  *   Limit: split_k * rows * n <= 1048512 floats, else SSD_ERR_OVERFLOW; bad shapes SSD_ERR_SHAPE; null
  *   pointers SSD_ERR_INVALID_ARG.
  * The first call on each device page-locks and maps the library's page of error words; under the driver's

@@ -54,6 +54,7 @@ struct TcParams {
   int two_sm;      // the CTAs of tiles 2i, 2i + 1 issue ONE tcgen05.mma.cta_group::2 (M = 256): each holds half of the activation tile
   uint32_t tmem_cols;
   float* out;
+  int out_vec;     // rows of `out` start on 16-byte boundaries: four features to a store.  (A caller's array may begin at any float.)
   bf16* act;
   int act_pitch;
   float* tile_max;
@@ -422,7 +423,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ 
       // Transpose 32 rows x 128 features through shared memory so that a thread stores four
       // consecutive features of one row: 8 vector stores per thread and chunk instead of 32 scalars.
       const int n_base = tile * kTileM;
-      const bool vec_ok = ((p.N & 3) == 0) && (n_base + kTileM <= p.N);
+      const bool vec_ok = p.out_vec && (n_base + kTileM <= p.N);
       for (int c0 = 32 * group; c0 < p.npad; c0 += 32 * kEpiGroups) {
         float v[32];
         if (n_kb > 0) tmem_ld32(taddr + c0, v);
@@ -624,7 +625,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ 
     auto store = [&](int row, const float4& acc) {
       if (!resid) {
         float* dst = p.out + (size_t)(row0 + row) * p.N + n_base + f4;
-        if ((p.N & 3) == 0) {
+        if (p.out_vec) {
           if (col_ok) *reinterpret_cast<float4*>(dst) = acc;
         } else {
           const float v[4] = {acc.x, acc.y, acc.z, acc.w};
@@ -810,6 +811,7 @@ int launch_gemm_tc(cudaStream_t st, const GemmArgs& g) {
   if (stages < 2) stages = 2;
   p.stages = stages;
   p.out = g.out; p.act = g.act; p.act_pitch = g.act_pitch;
+  p.out_vec = (((uintptr_t)g.out) & 15) == 0 && (g.N & 3) == 0;
   p.tile_max = g.tile_max; p.tile_sum = g.tile_sum; p.tile_arg = g.tile_arg;
   p.wait_limit_ns = g.wait_limit_ns > 0 ? g.wait_limit_ns : kWaitLimitNs;
   p.starve_kb = g.starve_kb;
