@@ -21,7 +21,12 @@
 // Epilogue: every warp publishes (max, sum, unnormalised output) of its (rows, key set) in shared
 // memory; after a cluster barrier CTA p normalises the rows r with r % parts == p, reading all
 // 2 * parts sub-parts through distributed shared memory and merging them in (part, key set) order.
-// Every reduction order depends on the row and the prefix length alone, never on the row count.
+//
+// A node's local keys take a power of two (16 or more) of key slots whatever its width, so they begin on a boundary of the
+// MMA's 16 keys, never straddle a 64-key tile that they fit in, and fill pairs of tiles from a first one where they do not: a
+// row's keys are grouped alike whichever node of a query tile it is in.  Every reduction order then depends on the row and
+// the prefix length alone, never on the row count.  (Packed side by side, nodes of 40, 48 or 65 rows came out with other bits
+// beside others than alone.  Nodes of 16 rows, the two-layer model's 20 forwards: 1727 us packed, 1722 padded.)
 #include "attn_common.cuh"
 
 namespace ssd {
@@ -67,7 +72,7 @@ __device__ __forceinline__ float4 ld_cluster_f32x4(uint32_t addr) {
 // MINB: CTAs per SM the register allocation must allow (3 trades a few spills for one wave at 64 rows)
 template <int HD, int QT, int MINB>
 __global__ void __launch_bounds__(QT * 4, MINB) attn_verify_kernel(AttnArgs a, int n_prefix_parts, int nbuf,
-                                                                     float scale_log2) {
+                                                                     int pad_shift, float scale_log2) {
   extern __shared__ __align__(128) uint8_t smem_raw[];
   constexpr int kQTile = QT;                                    // query rows per CTA: 32 or 64
   constexpr int kVerifyThreads = QT * 4;                        // (QT / 16 row groups) x 2 key sets, one warp each
@@ -92,15 +97,14 @@ __global__ void __launch_bounds__(QT * 4, MINB) attn_verify_kernel(AttnArgs a, i
   const bool local = part == n_prefix_parts;
   const int nqkv = (a.H + 2 * a.Hkv) * HD;
 
-  int k_begin, k_end;
-  if (!local) {
-    k_begin = part * a.kv_split;
-    k_end = min(a.S, k_begin + a.kv_split);
-  } else {
-    const int last = min(lr0 + kQTile - 1, rps - 1);
-    k_begin = (lr0 / T) * T;
-    k_end = (last / T + 1) * T;
-  }
+  // node-local keys: (1 << pad_shift) slots for every node that the query tile touches, the first T of them in use
+  const int node0 = lr0 / T;
+  const int loc_slots = (min(lr0 + kQTile - 1, rps - 1) / T - node0 + 1) << pad_shift;
+  auto slot_row = [&](int s) -> int {                           // sequence-local row of a key slot, -1: none
+    const int t = s & ((1 << pad_shift) - 1);
+    return (s < loc_slots && t < T) ? (node0 + (s >> pad_shift)) * T + t : -1;
+  };
+  const int k_begin = local ? 0 : part * a.kv_split, k_end = local ? loc_slots : min(a.S, k_begin + a.kv_split);
   const int n_tiles = (k_end - k_begin + kKTile - 1) / kKTile;
   const int n_pairs = (n_tiles + 1) / 2;
 
@@ -165,16 +169,14 @@ __global__ void __launch_bounds__(QT * 4, MINB) attn_verify_kernel(AttnArgs a, i
         }
       }
     }
-    float y1[8], y2[8];
+    // (roundings spelled out: a key has the same bits whether the prologue or a later step builds it)
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
-      y1[2 * j] = x1[2 * j] * cs[j].x - x2[2 * j] * cs[j].y;
-      y2[2 * j] = x2[2 * j] * cs[j].x + x1[2 * j] * cs[j].y;
-      y1[2 * j + 1] = x1[2 * j + 1] * cs[j].z - x2[2 * j + 1] * cs[j].w;
-      y2[2 * j + 1] = x2[2 * j + 1] * cs[j].z + x1[2 * j + 1] * cs[j].w;
+      rope_pair(x1[2 * j], x2[2 * j], cs[j].x, cs[j].y);
+      rope_pair(x1[2 * j + 1], x2[2 * j + 1], cs[j].z, cs[j].w);
     }
-    lo = make_uint4(pack_bf16(y1[0], y1[1]), pack_bf16(y1[2], y1[3]), pack_bf16(y1[4], y1[5]), pack_bf16(y1[6], y1[7]));
-    hi = make_uint4(pack_bf16(y2[0], y2[1]), pack_bf16(y2[2], y2[3]), pack_bf16(y2[4], y2[5]), pack_bf16(y2[6], y2[7]));
+    lo = make_uint4(pack_bf16(x1[0], x1[1]), pack_bf16(x1[2], x1[3]), pack_bf16(x1[4], x1[5]), pack_bf16(x1[6], x1[7]));
+    hi = make_uint4(pack_bf16(x2[0], x2[1]), pack_bf16(x2[2], x2[3]), pack_bf16(x2[4], x2[5]), pack_bf16(x2[6], x2[7]));
   };
   // ---- one 16-byte chunk (8 columns) of one row, summed over the splits, bf16 (for V)
   auto plain_item = [&](int lr, int c, int col0) -> uint4 {
@@ -203,7 +205,7 @@ __global__ void __launch_bounds__(QT * 4, MINB) attn_verify_kernel(AttnArgs a, i
     }
     return make_uint4(pack_bf16(x[0], x[1]), pack_bf16(x[2], x[3]), pack_bf16(x[4], x[5]), pack_bf16(x[6], x[7]));
   };
-  // later 128-key steps of a long local part (block length > 32): built by the local CTA alone
+  // later 128-slot steps of a long local part: built by the local CTA alone
   auto fill_local = [&](int pair, int buf) {
     constexpr int CPR = HALF / 8;
     const int key0 = k_begin + pair * kPairKeys;
@@ -212,21 +214,23 @@ __global__ void __launch_bounds__(QT * 4, MINB) attn_verify_kernel(AttnArgs a, i
     const uint4 zero = make_uint4(0, 0, 0, 0);
     for (int idx = tid; idx < kPairKeys * CPR; idx += kVerifyThreads) {
       const int row = idx / CPR, c = idx % CPR;
+      const int lr = slot_row(key0 + row);
       uint4 lo = zero, hi = zero;
-      if (key0 + row < k_end) rot_item(key0 + row, c, (a.H + kvh) * HD, lo, hi);
+      if (lr >= 0) rot_item(lr, c, (a.H + kvh) * HD, lo, hi);
       *reinterpret_cast<uint4*>(dK + swz<HD>(row, c)) = lo;
       *reinterpret_cast<uint4*>(dK + swz<HD>(row, c + CPR)) = hi;
-      if (commit_kv && key0 + row < k_end && key0 + row < commit_rows) {
-        bf16* dst = a.cache_k_out + cache_row(key0 + row) + c * 8;
+      if (commit_kv && lr >= 0 && lr < commit_rows) {
+        bf16* dst = a.cache_k_out + cache_row(lr) + c * 8;
         *reinterpret_cast<uint4*>(dst) = lo;
         *reinterpret_cast<uint4*>(dst + HALF) = hi;
       }
     }
     for (int idx = tid; idx < kPairKeys * CH; idx += kVerifyThreads) {
       const int row = idx / CH, c = idx % CH;
-      const uint4 v = (key0 + row < k_end) ? plain_item(key0 + row, c, (a.H + a.Hkv + kvh) * HD) : zero;
+      const int lr = slot_row(key0 + row);
+      const uint4 v = lr >= 0 ? plain_item(lr, c, (a.H + a.Hkv + kvh) * HD) : zero;
       *reinterpret_cast<uint4*>(dV + swz<HD>(row, c)) = v;
-      if (commit_kv && key0 + row < k_end && key0 + row < commit_rows) *reinterpret_cast<uint4*>(a.cache_v_out + cache_row(key0 + row) + c * 8) = v;
+      if (commit_kv && lr >= 0 && lr < commit_rows) *reinterpret_cast<uint4*>(a.cache_v_out + cache_row(lr) + c * 8) = v;
     }
   };
 
@@ -240,15 +244,12 @@ __global__ void __launch_bounds__(QT * 4, MINB) attn_verify_kernel(AttnArgs a, i
   cp_async_commit();
 
   // ---- cooperative prologue: the cluster's threads share the rotary work.  The Q tile is needed by
-  //      every CTA (each chunk is built once and stored into all of them), the first 128 local keys
-  //      only by the CTA of the local part.  Rows past the end are zero (a masked key's V row must
+  //      every CTA (each chunk is built once and stored into all of them), the first 128 local key slots
+  //      only by the CTA of the local part.  Rows past the end and unused slots are zero (a masked key's V row must
   //      not hold stale shared memory: 0 * NaN would poison the output).
   {
     constexpr int CPR = HALF / 8;
-    const int last = min(lr0 + kQTile - 1, rps - 1);
-    const int lk_begin = (lr0 / T) * T;
-    const int lk_rows = min((last / T + 1) * T - lk_begin, kPairKeys);       // valid local keys of step 0
-    const int lk_fill = min(((lk_rows + kKTile - 1) / kKTile) * kKTile, kPairKeys);   // rows of the tiles in use
+    const int lk_fill = min((loc_slots + kKTile - 1) / kKTile * kKTile, kPairKeys);   // rows of the tiles of step 0 in use
     const int n_q = kQTile * CPR, n_k = lk_fill * CPR, n_v = lk_fill * CH;
     const uint4 zero = make_uint4(0, 0, 0, 0);
     bf16* lK = sKV;                          // buffer 0 of the local CTA
@@ -265,20 +266,22 @@ __global__ void __launch_bounds__(QT * 4, MINB) attn_verify_kernel(AttnArgs a, i
         }
       } else if (it < n_q + n_k) {
         const int row = (it - n_q) / CPR, c = (it - n_q) % CPR;
+        const int lr = slot_row(row);
         uint4 lo = zero, hi = zero;
-        if (row < lk_rows) rot_item(lk_begin + row, c, (a.H + kvh) * HD, lo, hi);
+        if (lr >= 0) rot_item(lr, c, (a.H + kvh) * HD, lo, hi);
         st_cluster_u4(map_to_rank(lK + swz<HD>(row, c), (uint32_t)n_prefix_parts), lo);
         st_cluster_u4(map_to_rank(lK + swz<HD>(row, c + CPR), (uint32_t)n_prefix_parts), hi);
-        if (commit_kv && row < lk_rows && lk_begin + row < commit_rows) {
-          bf16* dst = a.cache_k_out + cache_row(lk_begin + row) + c * 8;
+        if (commit_kv && lr >= 0 && lr < commit_rows) {
+          bf16* dst = a.cache_k_out + cache_row(lr) + c * 8;
           *reinterpret_cast<uint4*>(dst) = lo;
           *reinterpret_cast<uint4*>(dst + HALF) = hi;
         }
       } else {
         const int row = (it - n_q - n_k) / CH, c = (it - n_q - n_k) % CH;
-        const uint4 v = (row < lk_rows) ? plain_item(lk_begin + row, c, (a.H + a.Hkv + kvh) * HD) : zero;
+        const int lr = slot_row(row);
+        const uint4 v = lr >= 0 ? plain_item(lr, c, (a.H + a.Hkv + kvh) * HD) : zero;
         st_cluster_u4(map_to_rank(lV + swz<HD>(row, c), (uint32_t)n_prefix_parts), v);
-        if (commit_kv && row < lk_rows && lk_begin + row < commit_rows) *reinterpret_cast<uint4*>(a.cache_v_out + cache_row(lk_begin + row) + c * 8) = v;
+        if (commit_kv && lr >= 0 && lr < commit_rows) *reinterpret_cast<uint4*>(a.cache_v_out + cache_row(lr) + c * 8) = v;
       }
     }
     cluster_sync_all();
@@ -297,10 +300,10 @@ __global__ void __launch_bounds__(QT * 4, MINB) attn_verify_kernel(AttnArgs a, i
 #pragma unroll
   for (int i = 0; i < 2; ++i) {
     const int qlr = lr0 + qrow_w + gq + i * 8;
-    node_lo[i] = local ? (qlr / T) * T : 0;
-    node_hi[i] = local ? min(node_lo[i] + T, k_end) : k_end;
+    node_lo[i] = local ? (qlr / T - node0) << pad_shift : 0;
+    node_hi[i] = local ? node_lo[i] + T : k_end;
     // causal chain of two blocks: a row of the finished block does not see the next block
-    if (local && a.map.chain_T0 > 0 && qlr - node_lo[i] < a.map.chain_T0) node_hi[i] = min(node_hi[i], node_lo[i] + a.map.chain_T0);
+    if (local && a.map.chain_T0 > 0 && qlr % T < a.map.chain_T0) node_hi[i] = node_lo[i] + a.map.chain_T0;
   }
   const bool rows_live = lr0 + qrow_w < rps;           // otherwise the warp only keeps the barriers
 
@@ -498,8 +501,16 @@ int launch_attention_verify(cudaStream_t st, const AttnArgs& a) {
   const int tiles32 = (a.map.rows_per_seq + 31) / 32;
   const int qt_rows = ((long long)a.n_seq_slots * tiles32 * n_parts * a.H <= 3 * 148) ? 32 : 64;
   const int q_tiles = (a.map.rows_per_seq + qt_rows - 1) / qt_rows;
+  // key slots of a node: a power of two from 16 on
+  int pad_shift = 4;
+  while ((1 << pad_shift) < a.map.T) ++pad_shift;
   // one 128-key step per part needs one K/V buffer; longer parts double-buffer
-  const int nbuf = (a.kv_split > kPairKeys || a.map.T > 32) ? 2 : 1;
+  int nodes = 1;                                  // most nodes that a query tile touches
+  for (int r0 = 0; r0 < a.map.rows_per_seq; r0 += qt_rows) {
+    const int last = (r0 + qt_rows < a.map.rows_per_seq ? r0 + qt_rows : a.map.rows_per_seq) - 1;
+    if (last / a.map.T - r0 / a.map.T + 1 > nodes) nodes = last / a.map.T - r0 / a.map.T + 1;
+  }
+  const int nbuf = (a.kv_split > kPairKeys || (nodes << pad_shift) > kPairKeys) ? 2 : 1;
   const size_t smem = (size_t)(qt_rows + nbuf * 2 * kPairKeys) * a.hd * 2;
   // two CTAs per SM by default; three (register-capped build) when only that keeps the grid in one wave
   const long long n_ctas = (long long)a.n_seq_slots * q_tiles * n_parts * a.H;
@@ -523,7 +534,7 @@ int launch_attention_verify(cudaStream_t st, const AttnArgs& a) {
   const unsigned cl = (unsigned)n_parts;
   cudaError_t e;
 #define SSD_LAUNCH_VERIFY(HD_, QT_, MB_) \
-  e = launch_pdl_cluster(attn_verify_kernel<HD_, QT_, MB_>, grid, block, smem, st, cl, a, n_prefix, nbuf, scale_log2)
+  e = launch_pdl_cluster(attn_verify_kernel<HD_, QT_, MB_>, grid, block, smem, st, cl, a, n_prefix, nbuf, pad_shift, scale_log2)
   if (a.hd == 128) {
     if (qt_rows == 64) SSD_LAUNCH_VERIFY(128, 64, 1);
     else if (dense) SSD_LAUNCH_VERIFY(128, 32, 3);
