@@ -480,7 +480,9 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ 
           for (int q4 = 0; q4 < 4; ++q4) {
             const float4 g = *reinterpret_cast<const float4*>(scratch + rr * kEpiPitch + fg + q4 * 4);
             const float4 u = *reinterpret_cast<const float4*>(scratch + rr * kEpiPitch + 64 + fg + q4 * 4);
-            const float a0 = swiglu(g.x, u.x), a1 = swiglu(g.y, u.y), a2 = swiglu(g.z, u.z), a3 = swiglu(g.w, u.w);
+            float a0, a1, a2, a3;
+            swiglu2(g.x, g.y, u.x, u.y, a0, a1);
+            swiglu2(g.z, g.w, u.z, u.w, a2, a3);
             __nv_bfloat162 lo = __floats2bfloat162_rn(a0, a1), hi = __floats2bfloat162_rn(a2, a3);
             packed[q4 * 2] = *reinterpret_cast<uint32_t*>(&lo);
             packed[q4 * 2 + 1] = *reinterpret_cast<uint32_t*>(&hi);

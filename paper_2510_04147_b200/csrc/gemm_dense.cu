@@ -508,7 +508,7 @@ gemm_dense_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant
           if (n_base + col(c) >= p.N) continue;
           float a[32];
 #pragma unroll
-          for (int j = 0; j < 32; ++j) a[j] = swiglu(run[c][0][j], run[c][1][j]);
+          for (int j = 0; j < 32; j += 2) swiglu2(run[c][0][j], run[c][0][j + 1], run[c][1][j], run[c][1][j + 1], a[j], a[j + 1]);
           rows_to_buf(trans, lane, a);
           const int f = ((n_base + (col(c) & ~127)) >> 1) + (col(c) & 63) + lc4;
 #pragma unroll

@@ -9,17 +9,47 @@ typedef __nv_bfloat16 bf16;
 
 namespace ssd {
 
-// silu(g) * u.  The quotient is g times the approximate reciprocal with one residual correction (Markstein's theorem: the
-// correctly rounded quotient but for rare cases in the last place; worst error against fp64 2.3e-7, as with `/`).  Without
-// that operator's branch the elements of an epilogue overlap: 32 of them took 3700 clocks of a thread, two warps to a
-// scheduler.  Gate/up of d 4096, ffn 12288 41.8 -> 40.9 us at 128 rows, 76.4 -> 69.3 at 512, 101 -> 99 at 768.  Where e^-g
-// passes 2^126 the reciprocal is zero, and with a finite residual the result.
-__device__ __forceinline__ float swiglu(float g, float u) {
-  const float d = 1.f + expf(-g);
-  float r;
-  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(d));
-  const float q = __fmul_rn(g, r);
-  return __fmul_rn(__fmaf_rn(__fmaf_rn(-q, fminf(d, 0x1p126f), g), r, q), u);
+// Two floats in a register pair, worked on by one instruction (each half rounded as by the scalar form)
+__device__ __forceinline__ uint64_t pair_f32(float x, float y) {
+  uint64_t p;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(p) : "f"(x), "f"(y));
+  return p;
+}
+__device__ __forceinline__ void unpair_f32(uint64_t p, float& x, float& y) { asm("mov.b64 {%0, %1}, %2;" : "=f"(x), "=f"(y) : "l"(p)); }
+__device__ __forceinline__ uint64_t mul_f32x2(uint64_t a, uint64_t b) {
+  uint64_t d;
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+  return d;
+}
+__device__ __forceinline__ uint64_t fma_f32x2(uint64_t a, uint64_t b, uint64_t c) {
+  uint64_t d;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
+  return d;
+}
+
+// a = silu(g) * u, for two elements.  The quotient is g times the approximate reciprocal with one residual correction
+// (Markstein's theorem: the correctly rounded quotient but for rare cases in the last place).  Without the division operator's
+// branch the elements of an epilogue overlap: 32 of them took 3700 clocks of a thread, two warps to a scheduler.  Gate/up of d
+// 4096, ffn 12288 41.8 -> 40.9 us at 128 rows, 76.4 -> 69.3 at 512, 101 -> 99 at 768.
+// The values of `/` over all g: the reciprocal is taken of a sixteenth of the denominator, because 1 / (1 + e^-g) is subnormal
+// from g = -87.4 down and the instruction flushes those to zero; where the residual is not finite (g infinite, or a
+// denominator past the largest float), the uncorrected quotient is g or 0 already.  Element by element these three more
+// operations cost eight sequences of 32 rows 2 % of a generation (281.8 -> 288.2 ms); in pairs gate/up takes as long as without
+// them (35.3 / 35.3 us at 64 rows, 53.6 / 54.0 at 256, 82.8 / 81.3 at 512).
+__device__ __forceinline__ void swiglu2(float g0, float g1, float u0, float u1, float& a0, float& a1) {
+  const uint64_t g = pair_f32(g0, g1), minus1 = pair_f32(-1.f, -1.f);
+  const uint64_t nd = fma_f32x2(pair_f32(expf(-g0), expf(-g1)), minus1, minus1);        // -(1 + e^-g)
+  float d0, d1, r0, r1, e0, e1, q0, q1, v0, v1;
+  unpair_f32(mul_f32x2(nd, pair_f32(-0x1p-4f, -0x1p-4f)), d0, d1);
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r0) : "f"(d0));
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r1) : "f"(d1));
+  const uint64_t r = mul_f32x2(pair_f32(r0, r1), pair_f32(0x1p-4f, 0x1p-4f)), q = mul_f32x2(g, r), rest = fma_f32x2(q, nd, g);
+  unpair_f32(rest, e0, e1);
+  unpair_f32(q, q0, q1);
+  unpair_f32(fma_f32x2(rest, r, q), v0, v1);
+  v0 = fabsf(e0) <= 3.402823466e38f ? v0 : q0;
+  v1 = fabsf(e1) <= 3.402823466e38f ? v1 : q1;
+  unpair_f32(mul_f32x2(pair_f32(v0, v1), pair_f32(u0, u1)), a0, a1);
 }
 
 // ---------------------------------------------------------------- programmatic dependent launch
