@@ -62,7 +62,8 @@ typedef struct {
 
 /* Supported shapes: head_dim 64 or 128; d_model, d_ffn, n_heads*head_dim multiples of 8;
  * n_heads a multiple of n_kv_heads; block_len <= 256.  `cuda_stream` is a cudaStream_t (NULL =
- * legacy default stream).  Allocates everything the context will ever need. */
+ * legacy default stream).  Allocates everything the context will ever need, but for the logits that
+ * ssd_verify_forward hands out when asked (their buffer grows with the largest such call). */
 int ssd_create(const ssd_config* cfg, void* cuda_stream, ssd_ctx** out);
 void ssd_destroy(ssd_ctx* ctx);
 const char* ssd_last_error(const ssd_ctx* ctx);   /* ctx may be NULL: message of a failed create */

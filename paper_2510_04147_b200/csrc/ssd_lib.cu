@@ -68,7 +68,7 @@ struct ssd_ctx {
   uint8_t* node_masked = nullptr;
   float* logits = nullptr;
   size_t logits_elems = 0;
-  // acceptance-limit probe (allocated on first use): per-tile candidate lists of the LM head, the merged
+  // top-k forwards and the acceptance-limit probe: per-tile candidate lists of the LM head, the merged
   // top-k per row, the draft forward's top-k per block position, match counters
   float* tile_topv = nullptr;
   int* tile_topi = nullptr;
@@ -577,20 +577,6 @@ __global__ void refresh_rows_kernel(const int* seq_ids, BlockState s, int b, int
   out[p] = id;
 }
 
-// Buffers of the acceptance-limit probe; allocated the first time a top-k forward is asked for.
-int ensure_topk_buffers(ssd_ctx* c) {
-  if (c->tile_topv) return SSD_OK;
-  const size_t tiles = gemm_tiles(c->V);
-  ALLOC(c, c->tile_topv, tiles * c->R_dec * kLmTopKMax);
-  ALLOC(c, c->tile_topi, tiles * c->R_dec * kLmTopKMax);
-  ALLOC(c, c->topk_tok, (size_t)c->R_dec * kLmTopKMax);
-  ALLOC(c, c->topk_prob, (size_t)c->R_dec * kLmTopKMax);
-  ALLOC(c, c->draft_top, (size_t)c->cfg.max_batch * c->bs.stride * kLmTopKMax);
-  ALLOC(c, c->probe_counts, kLmTopKMax + 1);
-  CUDA_TRY(c, cudaStreamSynchronize(c->st));
-  return SSD_OK;
-}
-
 // round opening: the draft forward's top-k of every block position of every sequence
 __global__ void probe_store_kernel(const int* topk_tok, int* draft_top, const int* seq_map, int T, int stride,
                                    int slot_rows, int row_offset) {
@@ -793,6 +779,17 @@ int ssd_create(const ssd_config* cfg, void* cuda_stream, ssd_ctx** out) {
     ALLOC(c, c->tile_max, tiles * c->R_dec);
     ALLOC(c, c->tile_sum, tiles * c->R_dec);
     ALLOC(c, c->tile_arg, tiles * c->R_dec);
+    {
+      // One array for the lists of the top-k forwards and the probe (all multiples of kLmTopKMax words), here and not in the first
+      // such call, which its allocations held up by 2 to 170 ms.  A quarter of what a row takes in `partial`.
+      const size_t lists = tiles * c->R_dec * kLmTopKMax, rows = (size_t)c->R_dec * kLmTopKMax, drafts = (size_t)k.max_batch * 2 * k.block_len * kLmTopKMax;
+      ALLOC(c, c->tile_topv, 2 * (lists + rows + kLmTopKMax + 1) + drafts);
+      c->tile_topi = reinterpret_cast<int*>(c->tile_topv + lists);
+      c->topk_tok = c->tile_topi + lists;
+      c->topk_prob = reinterpret_cast<float*>(c->topk_tok + rows);
+      c->draft_top = reinterpret_cast<int*>(c->topk_prob + rows);
+      c->probe_counts = reinterpret_cast<unsigned long long*>(c->draft_top + drafts);
+    }
     ALLOC(c, c->tok, R);
     ALLOC(c, c->conf, R);
     ALLOC(c, c->node_ids, R);
@@ -1462,8 +1459,6 @@ int ssd_verify_forward_topk(ssd_ctx* c, int32_t batch, int32_t n_nodes, int32_t 
   if (k < 1 || k > kLmTopKMax) return fail(c, SSD_ERR_INVALID_ARG, "k %d outside [1, %d]", k, kLmTopKMax);
   int rc = flush_pending(c);
   if (rc) return rc;
-  rc = ensure_topk_buffers(c);
-  if (rc) return rc;
   const size_t R = (size_t)batch * n_nodes * T;
   if (R > (size_t)c->R_dec) return fail(c, SSD_ERR_OVERFLOW, "%zu rows exceed the capacity %d set by max_batch/max_drafts/block_len", R, c->R_dec);
   if (c->cache_len + T > c->cfg.max_seq) return fail(c, SSD_ERR_OVERFLOW, "cache %d + block %d exceeds max_seq", c->cache_len, T);
@@ -1496,9 +1491,7 @@ int ssd_probe_acceptance_limit(ssd_ctx* c, int32_t T, int32_t draft_len, int32_t
   if (!c) return SSD_ERR_INVALID_ARG;
   if (!out_matched || !out_steps) return fail(c, SSD_ERR_INVALID_ARG, "null argument");
   if (draft_len < 0 || k_max < 1 || k_max > kLmTopKMax) return fail(c, SSD_ERR_INVALID_ARG, "draft_len >= 0 and k_max in [1, %d]", kLmTopKMax);
-  int rc = ensure_topk_buffers(c);
-  if (rc) return rc;
-  rc = ssd_block_begin(c, T);
+  int rc = ssd_block_begin(c, T);
   if (rc) return rc;
   clear_flags(c);
   CUDA_TRY(c, cudaMemsetAsync(c->probe_counts, 0, (kLmTopKMax + 1) * sizeof(unsigned long long), c->st));
