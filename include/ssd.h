@@ -212,7 +212,8 @@ int ssd_rewind(ssd_ctx* ctx, int32_t length);
 /* The skinny projection kernel alone: out[r][n] = sum_k x[r][k] * w[n][k] with bf16 operands and
  * fp32 accumulation, split over `split_k` K ranges that are summed in order.  DEVICE pointers:
  * x [rows, k] bf16, w [n, k] bf16 (both on 16-byte boundaries), out [rows, n] fp32 (anywhere a float may
- * lie).  k a multiple of 8.  Test / tuning hook. */
+ * lie).  k a multiple of 8; split_k * rows * n at most the floats of the context's split-K workspace (row capacity times
+ * the widest of 16 d_model, 4 to 16 widths of the fused q|k|v output, 2 d_ffn), else SSD_ERR_OVERFLOW.  Test / tuning hook. */
 int ssd_gemm_bf16(ssd_ctx* ctx, const void* x_dev, const void* w_dev, float* out_dev,
                   int32_t rows, int32_t n, int32_t k, int32_t split_k);
 

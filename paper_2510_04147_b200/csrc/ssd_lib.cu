@@ -192,6 +192,8 @@ int auto_split_residual(int tiles, int k) {
 // QKV: its finishing pass reads every split's partial sums.  One CTA per SM against two, eight layers: 36 tiles (4 splits, not 8)
 // 1018 -> 1007 us at 32 rows, 1328 -> 1282 at 128, 1591 -> 1555 at 192; 96 tiles (1, not 3) 968 -> 980, 1248 -> 1228, 1543 -> 1522.
 int auto_split_qkv(int tiles, int k) { return capped_split(148 / tiles, k); }
+// ... and what its partial sums have room for (option split_k_qkv), two CTAs per SM
+int most_split_qkv(int tiles, int k) { return capped_split((2 * 148 + tiles / 2) / tiles, k); }
 
 // Prefix keys per attention part: a function of the prefix length (and the option) only.  The
 // verification forward merges the parts inside one cluster, so prefix parts + the local part <= 8.
@@ -761,7 +763,8 @@ int ssd_create(const ssd_config* cfg, void* cuda_stream, ssd_ctx** out) {
     ALLOC(c, c->sq, R * c->sq_stride);
     c->partial_row_floats = (size_t)kMaxSplit * d;
     if ((size_t)4 * c->nqkv > c->partial_row_floats) c->partial_row_floats = (size_t)4 * c->nqkv;
-    if ((size_t)c->split_qkv * c->nqkv > c->partial_row_floats) c->partial_row_floats = (size_t)c->split_qkv * c->nqkv;
+    const size_t most = (size_t)most_split_qkv(gemm_tiles(c->nqkv), d) * c->nqkv;
+    if (most > c->partial_row_floats) c->partial_row_floats = most;
     if ((size_t)2 * c->ffn_pad > c->partial_row_floats) c->partial_row_floats = (size_t)2 * c->ffn_pad;
     c->partial_elems = R * c->partial_row_floats;
     ALLOC(c, c->partial, c->partial_elems);
@@ -1544,7 +1547,8 @@ int ssd_gemm_bf16(ssd_ctx* c, const void* x_dev, const void* w_dev, float* out_d
   if (!c) return SSD_ERR_INVALID_ARG;
   if (!x_dev || !w_dev || !out_dev) return fail(c, SSD_ERR_INVALID_ARG, "null argument");
   if (rows < 1 || n < 1 || k < 8 || (k % 8) || split_k < 1 || split_k > 8) return fail(c, SSD_ERR_SHAPE, "bad GEMM shape");
-  if ((size_t)split_k * rows * n > c->partial_elems) return fail(c, SSD_ERR_OVERFLOW, "GEMM exceeds the workspace");
+  if ((size_t)split_k * rows * n > c->partial_elems)
+    return fail(c, SSD_ERR_OVERFLOW, "split_k * rows * n = %zu exceeds this context's limit of %zu", (size_t)split_k * rows * n, c->partial_elems);
   clear_flags(c);
   GemmArgs g{};
   g.x = (const bf16*)x_dev; g.w = (const bf16*)w_dev; g.R = rows; g.N = n; g.K = k; g.x_pitch = k; g.w_pitch = k;
