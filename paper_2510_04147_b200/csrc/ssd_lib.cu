@@ -81,6 +81,7 @@ struct ssd_ctx {
   // block's tokens and accept counts.  `flags` is the device's address of the error words.
   volatile int* h_mapped = nullptr;
   int* flags = nullptr;
+  bool in_flight = false;        // kernels that may raise an error word have been launched and not been waited for
   BlockState bs{};
 
   int batch = 0, prompt_len = 0, cache_len = -1, block_tokens = 0;
@@ -146,6 +147,12 @@ int fail(ssd_ctx* c, int code, const char* fmt, ...) {
     if (e_ != cudaSuccess)                                                                         \
       return fail((c), e_ == cudaErrorMemoryAllocation ? SSD_ERR_OOM : SSD_ERR_CUDA, "%s: %s", #expr, \
                   cudaGetErrorString(e_));                                                         \
+  } while (0)
+
+#define SSD_TRY(expr)                   \
+  do {                                  \
+    const int rc_ = (expr);             \
+    if (rc_ != SSD_OK) return rc_;      \
   } while (0)
 
 template <typename T>
@@ -237,6 +244,7 @@ struct Scope {
   Scope(ssd_ctx* c_, int fam_, double bytes_, int n_launches = 1, int sub_ = -1)
       : c(c_), fam(fam_), sub(sub_), bytes(bytes_) {
     c->launches += n_launches;
+    c->in_flight = true;
     if (c->profiling) {
       cudaEventCreate(&e0);
       cudaEventCreate(&e1);
@@ -604,9 +612,21 @@ __global__ void probe_count_kernel(BlockState s, const int* draft_top, int n_slo
   }
 }
 
-// (only while no kernel of the context is in flight)
-void clear_flags(ssd_ctx* c) {
+int wait_for_stream(ssd_ctx* c) {
+  CUDA_TRY(c, cudaStreamSynchronize(c->st));
+  c->in_flight = false;
+  return SSD_OK;
+}
+
+// The words are cleared by the host, behind whatever may still raise one: a call that failed half way has left forwards in
+// flight, whose words are not the next call's.
+int clear_flags(ssd_ctx* c) {
+  if (c->in_flight) {
+    const int rc = wait_for_stream(c);
+    if (rc) return rc;
+  }
   for (int i = 0; i < 4; ++i) c->h_mapped[i] = 0;
+  return SSD_OK;
 }
 
 int check_flags_after_sync(ssd_ctx* c) {
@@ -616,8 +636,8 @@ int check_flags_after_sync(ssd_ctx* c) {
 }
 
 int sync_and_check(ssd_ctx* c) {
-  CUDA_TRY(c, cudaStreamSynchronize(c->st));
-  return check_flags_after_sync(c);
+  const int rc = wait_for_stream(c);
+  return rc ? rc : check_flags_after_sync(c);
 }
 
 // The commit forward of a finished block on its own (Section 3.2.4 leaves open how a block's K/V
@@ -625,7 +645,7 @@ int sync_and_check(ssd_ctx* c) {
 int commit_now(ssd_ctx* c, const int* ids, int stride, int T) {
   const int B = c->batch;
   CUDA_TRY(c, cudaMemcpy2DAsync(c->node_ids, T * sizeof(int), ids, stride * sizeof(int), T * sizeof(int), B, cudaMemcpyDeviceToDevice, c->st));
-  clear_flags(c);
+  SSD_TRY(clear_flags(c));
   RowMap map{T, T, c->cache_len, 0, nullptr};
   int rc = forward(c, FWD_FILL, c->node_ids, B * T, map, B, false, nullptr);
   if (rc) return rc;
@@ -904,7 +924,7 @@ int ssd_prefill_dev(ssd_ctx* c, int32_t batch, int32_t prompt_len, const int32_t
   if (batch < 1 || batch > c->cfg.max_batch) return fail(c, SSD_ERR_OVERFLOW, "batch %d outside [1, %d]", batch, c->cfg.max_batch);
   if (prompt_len < 1 || prompt_len > c->cfg.max_seq) return fail(c, SSD_ERR_OVERFLOW, "prompt_len %d outside [1, %d]", prompt_len, c->cfg.max_seq);
   if (!all_loaded(c)) return fail(c, SSD_ERR_STATE, "not every weight tensor has been loaded");
-  clear_flags(c);
+  SSD_TRY(clear_flags(c));
   // as many sequences per forward as the row capacity holds: their rows share one stream of the weights
   const int group = std::max(1, c->R_cap / prompt_len);
   for (int b = 0; b < batch; b += group) {
@@ -1117,7 +1137,7 @@ int step_enqueue(ssd_ctx* c, int md, bool* launched, const ProbeStep* probe = nu
     } else {
       const int frc = flush_pending(c);
       if (frc) return frc;
-      clear_flags(c);
+      SSD_TRY(clear_flags(c));
     }
   }
   // The window [this block | next block]: whenever a sequence can no longer fill its chain from this block.
@@ -1183,8 +1203,7 @@ int step_enqueue(ssd_ctx* c, int md, bool* launched, const ProbeStep* probe = nu
 
 // Waits for everything enqueued, checks the error flags and refreshes the host's mirror of `remaining`.
 int step_collect(ssd_ctx* c, int32_t* accepted, int32_t* n_nodes) {
-  CUDA_TRY(c, cudaStreamSynchronize(c->st));
-  const int rc = check_flags_after_sync(c);
+  const int rc = sync_and_check(c);
   if (rc) return rc;
   // (the acceptance kernel of the latest step wrote the words of every sequence that took part; a finished one's mirror
   // on the host stays as it is)
@@ -1213,7 +1232,7 @@ int ssd_block_step(ssd_ctx* c, int32_t max_drafts, int32_t* accepted, int32_t* n
   const int B = c->batch;
   if (accepted) memset(accepted, 0, B * sizeof(int));
   if (n_nodes) memset(n_nodes, 0, B * sizeof(int));
-  clear_flags(c);
+  SSD_TRY(clear_flags(c));
   bool launched = false;
   int rc = step_enqueue(c, md, &launched);
   if (rc) return rc;
@@ -1301,7 +1320,7 @@ int ssd_decode_block(ssd_ctx* c, int32_t mode, int32_t T, int32_t* out_tokens, i
   int rc = ssd_block_begin(c, T);
   if (rc) return rc;
   const int md = resolve_drafts(c, mode == SSD_MODE_STEPWISE ? 0 : -1);
-  clear_flags(c);
+  SSD_TRY(clear_flags(c));
   // A forward accepts between 1 and nodes tokens per sequence, so after it at least remaining - nodes
   // positions are still masked.  While that bound leaves every sequence a full chain (>= md + 1), the
   // next forward's launch shape is known without its predecessor's result: it is enqueued at once and
@@ -1323,7 +1342,7 @@ int ssd_decode_block(ssd_ctx* c, int32_t mode, int32_t T, int32_t* out_tokens, i
     }
     rc = step_collect(c, nullptr, nullptr);
     if (rc) return rc;
-    clear_flags(c);
+    SSD_TRY(clear_flags(c));
   }
   rc = ssd_block_commit(c);
   if (rc) return rc;
@@ -1356,7 +1375,7 @@ int ssd_verify_forward(ssd_ctx* c, int32_t batch, int32_t n_nodes, int32_t T, co
     if (node_ids[i] < 0 || node_ids[i] >= c->V) return fail(c, SSD_ERR_INVALID_ARG, "node id outside the vocabulary");
   CUDA_TRY(c, cudaMemcpyAsync(c->node_ids, node_ids, R * sizeof(int), cudaMemcpyHostToDevice, c->st));
   CUDA_TRY(c, cudaMemcpyAsync(c->node_masked, node_masked, R, cudaMemcpyHostToDevice, c->st));
-  clear_flags(c);
+  SSD_TRY(clear_flags(c));
   RowMap map{n_nodes * T, T, c->cache_len, 0, nullptr};
   LayerRange range;
   if (c->dual_total > 0) {
@@ -1440,7 +1459,7 @@ int ssd_verify_layers(ssd_ctx* c, int32_t batch, int32_t n_nodes, int32_t T, int
   if (R > (size_t)c->R_dec) return fail(c, SSD_ERR_OVERFLOW, "%zu rows exceed the capacity %d set by max_batch/max_drafts/block_len", R, c->R_dec);
   if (c->cache_len + T > c->cfg.max_seq) return fail(c, SSD_ERR_OVERFLOW, "cache %d + block %d exceeds max_seq", c->cache_len, T);
   CUDA_TRY(c, cudaMemcpyAsync(c->h, h_in, R * c->d * sizeof(float), cudaMemcpyHostToDevice, c->st));
-  clear_flags(c);
+  SSD_TRY(clear_flags(c));
   RowMap map{n_nodes * T, T, c->cache_len, 0, nullptr};
   LayerRange range;
   range.begin = layer_begin; range.end = layer_end; range.from_stream = true; range.lm_head = out_tok || out_conf;
@@ -1469,7 +1488,7 @@ int ssd_verify_forward_topk(ssd_ctx* c, int32_t batch, int32_t n_nodes, int32_t 
     if (node_ids[i] < 0 || node_ids[i] >= c->V) return fail(c, SSD_ERR_INVALID_ARG, "node id outside the vocabulary");
   CUDA_TRY(c, cudaMemcpyAsync(c->node_ids, node_ids, R * sizeof(int), cudaMemcpyHostToDevice, c->st));
   CUDA_TRY(c, cudaMemcpyAsync(c->node_masked, node_masked, R, cudaMemcpyHostToDevice, c->st));
-  clear_flags(c);
+  SSD_TRY(clear_flags(c));
   RowMap map{n_nodes * T, T, c->cache_len, 0, nullptr};
   LayerRange range;
   range.topk = k;
@@ -1496,7 +1515,7 @@ int ssd_probe_acceptance_limit(ssd_ctx* c, int32_t T, int32_t draft_len, int32_t
   if (draft_len < 0 || k_max < 1 || k_max > kLmTopKMax) return fail(c, SSD_ERR_INVALID_ARG, "draft_len >= 0 and k_max in [1, %d]", kLmTopKMax);
   int rc = ssd_block_begin(c, T);
   if (rc) return rc;
-  clear_flags(c);
+  SSD_TRY(clear_flags(c));
   CUDA_TRY(c, cudaMemsetAsync(c->probe_counts, 0, (kLmTopKMax + 1) * sizeof(unsigned long long), c->st));
   // stepwise decoding (every sequence accepts exactly one token per forward, so all stay in lockstep) in rounds
   // of draft_len + 1 forwards; nothing depends on a forward's result, so the whole block is enqueued at once
@@ -1524,7 +1543,7 @@ int ssd_refresh_cache(ssd_ctx* c) {
   if (c->dual_total <= 0) return fail(c, SSD_ERR_STATE, "the dual cache is off (option dual_cache)");
   const int T = c->in_block ? c->block_tokens : 0;
   if (c->cache_len + T > c->dual_total) return fail(c, SSD_ERR_OVERFLOW, "the sequence is longer than the dual cache's length %d", c->dual_total);
-  clear_flags(c);
+  SSD_TRY(clear_flags(c));
   for (int b = 0; b < c->batch; ++b) {
     const int rc = refresh_sequence(c, b, T);
     if (rc) return rc;
@@ -1549,7 +1568,7 @@ int ssd_gemm_bf16(ssd_ctx* c, const void* x_dev, const void* w_dev, float* out_d
   if (rows < 1 || n < 1 || k < 8 || (k % 8) || split_k < 1 || split_k > 8) return fail(c, SSD_ERR_SHAPE, "bad GEMM shape");
   if ((size_t)split_k * rows * n > c->partial_elems)
     return fail(c, SSD_ERR_OVERFLOW, "split_k * rows * n = %zu exceeds this context's limit of %zu", (size_t)split_k * rows * n, c->partial_elems);
-  clear_flags(c);
+  SSD_TRY(clear_flags(c));
   GemmArgs g{};
   g.x = (const bf16*)x_dev; g.w = (const bf16*)w_dev; g.R = rows; g.N = n; g.K = k; g.x_pitch = k; g.w_pitch = k;
   // (the splits of a tile are one cluster and sum their parts on chip)
