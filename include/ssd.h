@@ -231,7 +231,7 @@ int ssd_gemm_bf16(ssd_ctx* ctx, const void* x_dev, const void* w_dev, float* out
  * The first call on each device page-locks and maps the library's page of error words; under the driver's
  * lazy module loading that is also when the kernels are placed on the device, so make that first call early -
  * before the host's arena takes the remaining memory and before starting any stream capture.  Later calls
- * take no device memory at all.  Calls on different streams or threads may overlap.
+ * take no device memory at all.  Calls on different streams or threads may overlap, the first ones among them.
  * Synchronises the stream before returning; same result as ssd_gemm_bf16. */
 int ssd_gemm_bf16_noalloc(const void* x_dev, const void* w_dev, float* out_dev, int32_t rows, int32_t n,
                           int32_t k, int32_t split_k, void* cuda_stream);

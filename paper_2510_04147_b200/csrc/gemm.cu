@@ -21,6 +21,8 @@
 #include <math.h>
 #include <stdio.h>
 
+#include <atomic>
+
 namespace ssd {
 
 int gemm_tiles(int N) { return (N + 127) / 128; }
@@ -728,7 +730,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ 
 typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
                                   const cuuint64_t*, const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave,
                                   CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
-EncodeTiledFn g_encode = nullptr;
+std::atomic<EncodeTiledFn> g_encode{nullptr};       // (first calls of several threads may resolve it together)
 
 // [rows][pitch] bf16, K contiguous; box = 64 x box_rows; out-of-range elements read as zero
 bool make_tmap(CUtensorMap* m, const void* ptr, uint64_t rows, uint64_t cols, uint64_t pitch_elems, uint32_t box_rows) {
@@ -736,7 +738,7 @@ bool make_tmap(CUtensorMap* m, const void* ptr, uint64_t rows, uint64_t cols, ui
   cuuint64_t strides[1] = {pitch_elems * 2};
   cuuint32_t box[2] = {(cuuint32_t)kBlockK, box_rows};
   cuuint32_t estr[2] = {1, 1};
-  const CUresult r = g_encode(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void*>(ptr), dims, strides, box, estr,
+  const CUresult r = g_encode.load()(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void*>(ptr), dims, strides, box, estr,
                               CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
                               CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
   return r == CUDA_SUCCESS;
@@ -758,7 +760,7 @@ int encode_tmap_bf16_3d(void* map_out, const void* base, uint64_t cols, uint64_t
   cuuint64_t strides[2] = {row_pitch * 2, plane_pitch * 2};
   cuuint32_t box[3] = {(cuuint32_t)kBlockK, box_rows, 1};
   cuuint32_t estr[3] = {1, 1, 1};
-  return g_encode(reinterpret_cast<CUtensorMap*>(map_out), CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(base), dims, strides,
+  return g_encode.load()(reinterpret_cast<CUtensorMap*>(map_out), CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(base), dims, strides,
                   box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
                   CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS ? 0 : -4;
 }
@@ -838,7 +840,7 @@ int launch_gemm_tc(cudaStream_t st, const GemmArgs& g) {
   }
   if (!make_tmap(&tmX, g.x, (uint64_t)g.R, (uint64_t)g.K, (uint64_t)g.x_pitch, (uint32_t)(p.two_sm ? p.npad / 2 : p.npad))) return -4;
   // the opt-in to more than 48 KB of dynamic shared memory is a per-device attribute of the function
-  static bool smem_set[kMaxDevices] = {};
+  static std::atomic<bool> smem_set[kMaxDevices] = {};
   const int dev = device_slot();
   if (dev < 0) return -4;
   if (!smem_set[dev]) {

@@ -9,6 +9,7 @@
 // array in the library image, a summing kernel and a copy of the error word - 32 us for a call of 8 x 256 x 256, 42 us
 // for 77 x 4100 x 3592 in three splits.)
 #include "../../include/ssd.h"
+#include "error_words.h"
 #include "kernels.h"
 
 #include <atomic>
@@ -22,7 +23,7 @@ constexpr int kMaxDevices = 64;
 // Error words of the calls in flight, one page of this library's own memory, page-locked and mapped on first use.
 constexpr int kErrWords = 1024;
 alignas(4096) int g_err_words[kErrWords];
-std::atomic<unsigned> g_err_next{0};
+ssd::ErrorWords<kErrWords> g_err_loans;
 
 std::mutex g_setup_mutex;
 std::atomic<int*> g_err_dev[kMaxDevices] = {};               // the page's address on each device
@@ -56,12 +57,15 @@ extern "C" int ssd_gemm_bf16_noalloc(const void* x_dev, const void* w_dev, float
   int* const err_dev = err_words_on_current_device();
   if (!err_dev) return SSD_ERR_CUDA;
   cudaStream_t st = reinterpret_cast<cudaStream_t>(cuda_stream);
-  const unsigned slot = g_err_next.fetch_add(1) % kErrWords;   // (a call has left its word before 1024 later ones have begun)
-  volatile int* word = g_err_words + slot;
+  struct Loan {
+    const int slot = g_err_loans.borrow();
+    ~Loan() { g_err_loans.give_back(slot); }
+  } const loan;
+  volatile int* word = g_err_words + loan.slot;
   *word = 0;
   ssd::GemmArgs g{};
   g.x = (const bf16*)x_dev; g.w = (const bf16*)w_dev; g.R = rows; g.N = n; g.K = k; g.x_pitch = k; g.w_pitch = k;
-  g.splits = split_k; g.epi = split_k > 1 ? ssd::EPI_SUM : ssd::EPI_PARTIAL; g.out = out_dev; g.err_flag = err_dev + slot;
+  g.splits = split_k; g.epi = split_k > 1 ? ssd::EPI_SUM : ssd::EPI_PARTIAL; g.out = out_dev; g.err_flag = err_dev + loan.slot;
   g.plain_launch = 1;
   const int rc = ssd::launch_gemm_tc(st, g);
   if (rc != 0) return rc;
