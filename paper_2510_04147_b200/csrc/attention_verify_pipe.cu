@@ -5,7 +5,7 @@
 // 0, visibility per row: the row's own node, block-causal inside a chain of two blocks) followed by the cached keys in
 // 128-key tiles (under the dual cache: the keys before the hole, then those behind it).  q, k and v come rotated and
 // rounded from the projection's epilogue, so every tile is a tensor-map copy; rows past the end of the cached keys are
-// out of the map's bounds and arrive as zeros.  A node's local keys take a power of two (16 or more) of key slots whatever
+// out of the map's bounds and arrive as zeros, as do those past the end of a node.  A node's local keys take a power of two (16 or more) of key slots whatever
 // its width: the tensor core takes keys in groups of 16 and the sums below are a binary tree over those, so a row's bits
 // do not depend on which node of a tile it is in.
 //
@@ -253,7 +253,7 @@ attn_verify_pipe_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
   const int kvh = h / (a.H / a.Hkv);
   const int lr0 = qt * tile_rows;
   const size_t grow0 = (size_t)slot * rps + lr0;
-  const int rows_here = min(tile_rows, rps - lr0), nodes_here = rows_here / T;
+  const int rows_here = min(tile_rows, rps - lr0), nodes_here = rows_here / T, node0 = (int)grow0 / T;     // (nodes of all sequences)
   // this CTA's tiles: global tile index first + u, u = 0 .. n_tiles - 1
   const int first = part * g.n_all / g.n_parts, n_tiles = (part + 1) * g.n_all / g.n_parts - first;
 
@@ -268,7 +268,8 @@ attn_verify_pipe_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
   }
   if (first == 0 && tid < kPipeThreads) {
-    // the V rows of tile 0 behind the nodes' slots: zero (a masked key's V row must be finite: 0 * NaN would poison O)
+    // the V rows of tile 0 behind the nodes' slots: zero (a masked key's V row must be finite: 0 * NaN would poison O).  So are a
+    // node's own unused slots: a plane of the map is one node, what its box takes beyond arrives as zeros
     for (int idx = nodes_here * g.t_pad * 16 + tid; idx < kKeys * 16; idx += kPipeThreads)
       *reinterpret_cast<uint4*>(sVs + tile_off(idx >> 4, idx & 15)) = make_uint4(0, 0, 0, 0);
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
@@ -351,7 +352,7 @@ attn_verify_pipe_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
           mbar_arrive_expect_tx(bar, (uint32_t)(nodes_here * g.t_pad * 256));
           for (int n = 0; n < nodes_here; ++n)
             for (int half = 0; half < 2; ++half)
-              tma_load_2d(dst + half * kHalfBytes + n * g.t_pad * 128, &tmLK, bar, kvh * kHD + half * 64, (int)grow0 + n * T);
+              tma_load_3d(dst + half * kHalfBytes + n * g.t_pad * 128, &tmLK, bar, kvh * kHD + half * 64, 0, node0 + n);
         } else {
           const int r = gt <= g.n_a ? (gt - 1) * kKeys : g.row_b + (gt - 1 - g.n_a) * kKeys;
           const int plane = seq_of_slot(a.map, slot) * a.Hkv + kvh;
@@ -367,7 +368,7 @@ attn_verify_pipe_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
           mbar_arrive_expect_tx(bar, (uint32_t)(nodes_here * g.t_pad * 256));
           for (int n = 0; n < nodes_here; ++n)
             for (int half = 0; half < 2; ++half)
-              tma_load_2d(dst + half * kHalfBytes + n * g.t_pad * 128, &tmLV, bar, kvh * kHD + half * 64, (int)grow0 + n * T);
+              tma_load_3d(dst + half * kHalfBytes + n * g.t_pad * 128, &tmLV, bar, kvh * kHD + half * 64, 0, node0 + n);
         } else {
           const int r = gt <= g.n_a ? (gt - 1) * kKeys : g.row_b + (gt - 1 - g.n_a) * kKeys;
           const int plane = seq_of_slot(a.map, slot) * a.Hkv + kvh;
@@ -703,8 +704,8 @@ int launch_attention_verify_pipe(cudaStream_t st, const AttnArgs& a, int n_parts
   const uint64_t bound = (uint64_t)(a.S + a.hole_len > 0 ? a.S + a.hole_len : 1);
   const uint64_t qw = (uint64_t)a.H * kHD, kw = (uint64_t)a.Hkv * kHD;
   if (encode_tmap_bf16_2d(&tm[0], a.q, (uint64_t)a.R, qw, qw, (uint32_t)qt_rows) != 0 ||
-      encode_tmap_bf16_2d(&tm[1], a.local_k, (uint64_t)a.R, kw, kw, (uint32_t)g.t_pad) != 0 ||
-      encode_tmap_bf16_2d(&tm[2], a.local_v, (uint64_t)a.R, kw, kw, (uint32_t)g.t_pad) != 0 ||
+      encode_tmap_bf16_3d(&tm[1], a.local_k, kw, (uint64_t)T, (uint64_t)(a.R / T), kw, kw * T, (uint32_t)g.t_pad) != 0 ||
+      encode_tmap_bf16_3d(&tm[2], a.local_v, kw, (uint64_t)T, (uint64_t)(a.R / T), kw, kw * T, (uint32_t)g.t_pad) != 0 ||
       encode_tmap_bf16_3d(&tm[3], a.cache_k, kHD, bound, planes, kHD, a.kv_head_stride, kKeys) != 0 ||
       encode_tmap_bf16_3d(&tm[4], a.cache_v, kHD, bound, planes, kHD, a.kv_head_stride, kKeys) != 0)
     return -4;
