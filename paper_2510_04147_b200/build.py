@@ -2,6 +2,7 @@
 from __future__ import annotations
 
 import os
+import re
 import subprocess
 import sys
 from concurrent.futures import ThreadPoolExecutor
@@ -24,6 +25,18 @@ def _newer(src: str, dst: str) -> bool:
     return any(os.path.getmtime(d) > t for d in deps)
 
 
+def check_register_shares(source: str, log: str) -> None:
+    """Raises if a kernel of `source` that shifts registers between its warpgroups (kRegsSoftmax, kRegsOther) was compiled to fewer
+    than the shares add up to: they come out of what a block is launched with, so its launcher would refuse every launch."""
+    const = {k: int(v) for k, v in re.findall(r"(kThreads|kRegsSoftmax|kRegsOther) = (\d+)", source)}
+    if "kRegsSoftmax" not in const:
+        return
+    need = 256 * const["kRegsSoftmax"] + (const["kThreads"] - 256) * const["kRegsOther"]
+    used = [int(n) for n in re.findall(r"Used (\d+) registers", log)]
+    if not used or min(used) * const["kThreads"] < need:
+        raise RuntimeError(f"register shares of {need} need {-(-need // const['kThreads'])} registers a thread, compiled to {used}")
+
+
 def build(force: bool = False, verbose: bool = False) -> str:
     nvcc = os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc")
     os.makedirs(OBJ, exist_ok=True)
@@ -36,6 +49,12 @@ def build(force: bool = False, verbose: bool = False) -> str:
         r = subprocess.run([nvcc, *NVCC_FLAGS, "-c", src, "-o", obj], capture_output=True, text=True)
         if r.returncode != 0:
             raise RuntimeError(f"nvcc failed on {name}:\n{r.stdout}\n{r.stderr}")
+        try:
+            with open(src) as f:
+                check_register_shares(f.read(), r.stderr)
+        except RuntimeError:
+            os.remove(obj)                         # (or the next build would take it for a good one)
+            raise
         return obj, r.stderr
 
     with ThreadPoolExecutor(max_workers=len(SOURCES)) as ex:

@@ -419,7 +419,7 @@ int launch(cudaStream_t st, const AttnArgs& a, const CUtensorMap& tmQ, const CUt
     if (cudaFuncSetAttribute(attn_fill_tc_kernel<kQ>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess ||
         cudaFuncGetAttributes(&fa, attn_fill_tc_kernel<kQ>) != cudaSuccess)
       return -4;
-    // the warpgroups' shares come out of what the block is launched with
+    // the warpgroups' shares come out of what the block is launched with (the build refuses a compilation to fewer)
     if (fa.numRegs * kThreads < 256 * kRegsSoftmax + 128 * kRegsOther) return -4;
     attr_set[dev] = true;
   }
