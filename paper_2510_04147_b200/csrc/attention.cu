@@ -238,7 +238,7 @@ __global__ void __launch_bounds__(256) attn_merge_kernel(const float* part_o, co
 
 }  // namespace
 
-void launch_attention(cudaStream_t st, const AttnArgs& a, int* launches) {
+void launch_attention(cudaStream_t st, const AttnArgs& a) {
   const int n_prefix = (a.S + a.kv_split - 1) / a.kv_split;
   const int has_local = a.local_k != nullptr ? 1 : 0;
   const int n_parts = n_prefix + has_local;
@@ -250,7 +250,6 @@ void launch_attention(cudaStream_t st, const AttnArgs& a, int* launches) {
   dim3 mgrid(a.R, (a.H * a.hd / 2 + 255) / 256);
   launch_pdl(attn_merge_kernel, mgrid, dim3(256), 0, st, (const float*)a.part_o, (const float2*)a.part_ml, a.out, a.R,
              a.H, a.hd, n_parts);
-  if (launches) *launches += 2;
 }
 
 }  // namespace ssd

@@ -435,7 +435,7 @@ int launch(cudaStream_t st, const AttnArgs& a, const CUtensorMap& tmQ, const CUt
 int launch_attention_fill_tc(cudaStream_t st, const AttnArgs& a) {
   if (a.hd != kHD || a.kv_pos_stride != (size_t)kHD || a.cache_seq_stride != a.kv_head_stride * (size_t)a.Hkv || a.map.seq_map ||
       !a.err_flag || a.cache_rows == 0)
-    return 1;
+    return -2;
   alignas(64) CUtensorMap tmQ, tmK, tmV;
   const uint64_t planes = (uint64_t)a.cache_rows * kHD / a.kv_head_stride;       // (sequence, kv head) pairs
   if (encode_tmap_bf16_2d(&tmQ, a.q, (uint64_t)a.R, (uint64_t)a.H * kHD, (uint64_t)a.H * kHD, kTile) != 0 ||

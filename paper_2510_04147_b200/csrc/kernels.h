@@ -214,9 +214,9 @@ struct AttnArgs {
   int n_seq_slots;
 };
 // cache-fill form for head dimension 64
-void launch_attention(cudaStream_t st, const AttnArgs& a, int* launches);
+void launch_attention(cudaStream_t st, const AttnArgs& a);
 // The cache-fill form on the tcgen05 tensor cores (head dimension 128): reads a.q and the cache, writes a.out; slots are
-// consecutive sequences from map.seq_base.  Returns 0 (launched), 1 (shape not covered) or a negative ssd error code.
+// consecutive sequences from map.seq_base.  Returns 0 or a negative ssd error code.
 int launch_attention_fill_tc(cudaStream_t st, const AttnArgs& a);
 // Verification-forward form: one kernel; rotary embedding, node-local K/V and the merge of the
 // key parts (through a thread-block cluster) inside.  Needs prefix parts + 1 <= kAttnMaxClusterParts.

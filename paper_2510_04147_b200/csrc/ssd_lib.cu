@@ -491,9 +491,9 @@ int forward(ssd_ctx* c, int kind, const int* ids_dev, int R, RowMap map, int n_s
       Scope sc(c, SSD_PROF_ATTN, kvb, tc ? 1 : 2);
       if (tc) {
         const int arc = launch_attention_fill_tc(c->st, a);
-        if (arc != 0) return fail(c, arc < 0 ? arc : SSD_ERR_SHAPE, "cache-fill attention rejected %d rows (code %d)", R, arc);
+        if (arc != 0) return fail(c, arc, "cache-fill attention rejected %d rows (code %d)", R, arc);
       } else {
-        launch_attention(c->st, a, nullptr);
+        launch_attention(c->st, a);
       }
     } else {
       Scope sc(c, SSD_PROF_ATTN, kvb, 1);
