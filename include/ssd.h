@@ -274,8 +274,8 @@ int ssd_profile_read(ssd_ctx* ctx, int64_t* launches, double* milliseconds, doub
  *        evenly: it sets the number of parts (prefix / kv_split + 1, 2 to 8; automatic: 8 / 4 / 2 for up to 16 / 32 /
  *        more heads);
  *   "max_drafts" lower the draft-length cap below the capacity fixed at creation;
- *   "gemm_max_stages" tuning: cap on the depth of the projection kernel's shared-memory ring (0 = as deep as
- *        two CTAs per SM allow, the default); changes no result;
+ *   "gemm_max_stages" tuning: cap on the depth of the projection kernel's shared-memory ring (0, the default = as
+ *        deep as its shared memory allows: a whole SM's for launches of up to 148 CTAs, else half of it); changes no result;
  *   "wait_limit_us" bound of every device-side barrier wait of the projection kernel in microseconds (0 = the
  *        default of 2 s): when it runs out the kernel raises an error word, lets its copies in flight land,
  *        frees its tensor memory and returns, and the call reports SSD_ERR_TIMEOUT; the context stays usable;

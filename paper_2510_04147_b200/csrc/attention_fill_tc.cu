@@ -8,7 +8,8 @@
 //                          back as bf16 into the first half of S_i's columns)
 //     O_i += P_i V        (A operand from tensor memory, V as stored, [key][hd])
 // One warp issues all MMAs in the order PV_0(j), S_0(j+1), PV_1(j), S_1(j+1): while one warpgroup is in its
-// exponentials, the tensor core works for the other.  PV starts when the first 64 keys' P is written.  A warp asks the tensor-map engine for the K and V tiles two
+// exponentials, the tensor core works for the other.  (Two query tiles that take turns with the tensor core, P over the scores'
+// columns and the late rescale below are the published scheme of FlashAttention-4.)  PV starts when the first 64 keys' P is written.  A warp asks the tensor-map engine for the K and V tiles two
 // ahead; keys past the end of the sequence are out of the map's bounds and arrive as zeros.
 //
 // The bounds are the tensor core and the special-function unit alike: a query tile x key tile is 1024 clocks of MMA (two

@@ -499,7 +499,7 @@ int launch_attention_verify(cudaStream_t st, const AttnArgs& a) {
   const float scale_log2 = (1.0f / sqrtf((float)a.hd)) * 1.4426950408889634f;
   // 32-row query tiles (128 threads) while that still fits the machine in one wave, else 64-row tiles
   const int tiles32 = (a.map.rows_per_seq + 31) / 32;
-  const int qt_rows = ((long long)a.n_seq_slots * tiles32 * n_parts * a.H <= 3 * 148) ? 32 : 64;
+  const int qt_rows = ((long long)a.n_seq_slots * tiles32 * n_parts * a.H <= 3 * kSms) ? 32 : 64;
   const int q_tiles = (a.map.rows_per_seq + qt_rows - 1) / qt_rows;
   // key slots of a node: a power of two from 16 on
   int pad_shift = 4;
@@ -514,7 +514,7 @@ int launch_attention_verify(cudaStream_t st, const AttnArgs& a) {
   const size_t smem = (size_t)(qt_rows + nbuf * 2 * kPairKeys) * a.hd * 2;
   // two CTAs per SM by default; three (register-capped build) when only that keeps the grid in one wave
   const long long n_ctas = (long long)a.n_seq_slots * q_tiles * n_parts * a.H;
-  const bool dense = qt_rows == 32 && n_ctas > 2 * 148;
+  const bool dense = qt_rows == 32 && n_ctas > 2 * kSms;
   static bool attr_set[kMaxDevices] = {};        // the shared-memory opt-in is per device
   const int dev = device_slot();
   if (dev < 0) return -4;

@@ -27,7 +27,7 @@
 // Bound by the serial chain of a tile, not by bytes, except for long prefixes under small query tiles.  Of a 128-row tile's
 // 3400 clocks (clock64 at each step, 4096 keys) the scores' maximum took 580, the wait for O += P V 425, exponentials, sums and P
 // 1850, of which the special-function unit accounts for 1024.  Taken out: the visibility test of every key (masked scores become
-// -inf where they are loaded) and that wait: 4 sequences of 4096 keys 77 -> 69 us at 128 rows each, 1536 keys 24.2 -> 22.9.
+// -inf where they are loaded) and that wait: 4 sequences of 4096 keys 77 -> 72 us at 128 rows each, 1536 keys 24.2 -> 22.9.
 // Keeping all 64 scores of a thread in registers, four threads to a row, or even and odd tiles in two streams were no faster.
 // us per layer in the live stream (the forms before it, which summed and rotated the projection's split-K partials themselves, in
 // brackets; finishing q, k and v is now a pass of 3 to 10 us): one sequence, 512 keys, 32 / 64 / 128 rows 10 (15) / 13 (20) /

@@ -1,4 +1,4 @@
-// Device helpers shared by the two attention kernels: asynchronous copies, ldmatrix / mma.sync
+// Device helpers shared by the attention kernels: asynchronous copies, ldmatrix / mma.sync
 // wrappers and the XOR swizzle of a [rows][HD] bf16 tile in shared memory.
 #pragma once
 #include "kernels.h"

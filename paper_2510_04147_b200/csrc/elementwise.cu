@@ -338,7 +338,7 @@ void launch_convert_rows(cudaStream_t st, const void* src, int src_is_f32, bf16*
                          int group, int group_stride, int group_offset) {
   const size_t total = (size_t)rows * cols;
   int blocks = (int)((total + 255) / 256);
-  if (blocks > 148 * 16) blocks = 148 * 16;
+  if (blocks > kSms * 16) blocks = kSms * 16;
   if (blocks < 1) blocks = 1;
   convert_rows_kernel<<<blocks, 256, 0, st>>>(src, src_is_f32, dst, rows, cols, dst_pitch, group, group_stride,
                                               group_offset);
@@ -348,7 +348,7 @@ void launch_convert_tiled(cudaStream_t st, const void* src, int src_is_f32, bf16
                           int group, int group_stride, int group_offset) {
   const size_t total = (size_t)rows * cols;
   int blocks = (int)((total + 255) / 256);
-  if (blocks > 148 * 16) blocks = 148 * 16;
+  if (blocks > kSms * 16) blocks = kSms * 16;
   if (blocks < 1) blocks = 1;
   convert_tiled_kernel<<<blocks, 256, 0, st>>>(src, src_is_f32, dst, rows, cols, kb_total, group, group_stride,
                                                group_offset);

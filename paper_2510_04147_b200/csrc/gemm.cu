@@ -808,7 +808,7 @@ int launch_gemm_tc(cudaStream_t st, const GemmArgs& g) {
   // tiles of K 4096 as one CTA each (8 and 6 stages) take 20.9 and 22.7 us, as three splits of half the ring 19.2 and 22.8
   // with three partial sums instead of one for the finishing pass to read.
   const long long ctas = (long long)gemm_tiles(g.N) * g.splits * p.row_blocks;
-  const int budget = (ctas <= 148 ? 212 : 108) * 1024;
+  const int budget = (ctas <= kSms ? 212 : 108) * 1024;
   int stages = budget / stage_bytes;
   if (stages > kMaxStages) stages = kMaxStages;
   if (g.max_stages > 0 && stages > g.max_stages) stages = g.max_stages;

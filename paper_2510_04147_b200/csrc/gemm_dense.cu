@@ -19,13 +19,12 @@
 // K splits: a verification forward of few rows runs in gemm.cu, whose sums are cut into `splits` K ranges that are added
 // in order.  Here the ranges follow one another in one CTA: each is accumulated by itself and the epilogue threads
 // add it to a running sum in registers, in the same order with the same roundings - so a row's bits do not depend on the
-// number of rows, and it does not matter which kernel takes a forward.  (The cache-fill forward has its own rule, and one
-// range.)  Every wait is bounded as in gemm.cu.
+// number of rows, and it does not matter which kernel takes a forward.  Every wait is bounded as in gemm.cu.
 //
 // The bound is the tensor core (256 features: 0.31 us a K block under the power cap; 0.36 measured) and, for narrow tiles, the
 // shared memory it reads.  One warp issues the copies and one the MMAs, and both walk their loops converged with one elected
 // lane: with descriptors rebuilt in one lane's registers and divisions per K block, issuing took 580 clocks a K block and was
-// the bound at every size (down projection at 512 rows 79 us, now 49).
+// the bound at every size (down projection at 512 rows 79 us, now 53).
 // us per layer of the four projections, this kernel / gemm.cu (with its pass for q, k, v): d 4096, ffn 12288: 512 rows 202 / 242,
 // 1024 335 / 415, 4096 1530 / 2560; d 3584, ffn 18944: 512 rows 208 / 234, 4096 1620 / 2600.  By projection, and below that: where
 // the forward chooses.

@@ -111,6 +111,10 @@ inline cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, s
 }
 #endif
 
+// The rules that share work out are functions of the shape alone, so they take the machine's size from here; a grid of
+// persistent CTAs asks the device.
+constexpr int kSms = 148;
+
 // ---------------------------------------------------------------- per-device set-up
 // Function attributes (the opt-in to large dynamic shared memory) belong to a device, not to the
 // process: launchers keep one flag per device ordinal and set the attribute on a device's first use.
@@ -192,7 +196,7 @@ struct AttnArgs {
   bf16* cache_v_out;
   int* err_flag;              // word set non-zero when a bounded wait expires (tcgen05 form)
   const bf16* q;        // [R][H][hd], rotated
-  const bf16* cache_k;  // layer base: [seq][max_seq][Hkv][hd]
+  const bf16* cache_k;  // layer base: [seq][Hkv][max_seq][hd]
   const bf16* cache_v;
   const bf16* local_k;  // [R][Hkv][hd] or nullptr (no node-local keys)
   const bf16* local_v;
@@ -237,7 +241,7 @@ constexpr int kAttnTcMaxNode = 128;     // widest node of the tcgen05 form: its 
 // rmsnorm(h) * g . W^T  ==  inv_rms(row) * ((h * g) . W^T), with inv_rms from the sums of squares.
 // EPI_SUM: the same cluster reduction, the sums themselves go to `out` (fp32 [R][N]).
 // EPI_QKV (dense kernel only): rotary embedding of q and k, everything rounded to bf16; q rows to their buffer, k and v
-// rows to the cache.
+// rows to the node-local buffers, the cache or both.
 enum { EPI_PARTIAL = 0, EPI_SWIGLU = 1, EPI_LMHEAD = 2, EPI_RESIDUAL = 3, EPI_QKV = 4, EPI_SUM = 5 };
 constexpr int kGemmMaxClusterSplits = 8;
 constexpr int kLmTopKMax = 8;   // most candidates per row the LM-head epilogue can rank

@@ -193,14 +193,14 @@ int capped_split(int s, int k) {
 // A power of two: clusters of five leave so many SMs of a GPC unused that 140 CTAs take two waves (28 tiles: 1019 -> 1164 us).
 int auto_split_residual(int tiles, int k) {
   int s = 8;
-  while (s > 1 && tiles * s > 148) s >>= 1;
+  while (s > 1 && tiles * s > kSms) s >>= 1;
   return capped_split(s, k);
 }
 // QKV: its finishing pass reads every split's partial sums.  One CTA per SM against two, eight layers: 36 tiles (4 splits, not 8)
 // 1018 -> 1007 us at 32 rows, 1328 -> 1282 at 128, 1591 -> 1555 at 192; 96 tiles (1, not 3) 968 -> 980, 1248 -> 1228, 1543 -> 1522.
-int auto_split_qkv(int tiles, int k) { return capped_split(148 / tiles, k); }
+int auto_split_qkv(int tiles, int k) { return capped_split(kSms / tiles, k); }
 // ... and what its partial sums have room for (option split_k_qkv), two CTAs per SM
-int most_split_qkv(int tiles, int k) { return capped_split((2 * 148 + tiles / 2) / tiles, k); }
+int most_split_qkv(int tiles, int k) { return capped_split((2 * kSms + tiles / 2) / tiles, k); }
 
 // Prefix keys per attention part: a function of the prefix length (and the option) only.  The
 // verification forward merges the parts inside one cluster, so prefix parts + the local part <= 8.
@@ -413,6 +413,8 @@ int forward(ssd_ctx* c, int kind, const int* ids_dev, int R, RowMap map, int n_s
   //   O       17 / 20    20 / 20    21 / 20    25 / 20    28 / 20    30 / 21    42 / 32    45 / 32    49 / 33
   //   gate/up 55 / 61    60 / 55    74 / 90    88 / 92    95 / 93   102 / 86   120 / 130  133 / 130  147 / 126
   //   down    36 / 71    43 / 73    50 / 73    68 / 75    72 / 76    77 / 78   125 / 109  132 / 111  142 / 118
+  // (Where the two shapes disagree - down at 448 rows, gate/up at 640 - the line costs one of them up to 5 %; other widths take
+  // the same lines unmeasured.)
   const bool may = R > c->dense_rows;
   const bool dense_gu = may && (R <= 256 || R * 16 >= (R + 255) / 256 * 256 * 13);
   const bool dense_qkv = may && (R > 384 || (R <= 256 && gemm_tiles(c->nqkv) >= 74));

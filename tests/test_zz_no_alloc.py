@@ -1,7 +1,7 @@
 """The allocation-free projection entry point, for hosts that cannot call cudaMalloc while running
 (a process whose device memory all belongs to its own arena, or a loop that may not block or fail on
-an allocation).  It must give what the context-based entry point gives, call after call, although
-all calls share one fixed scratch array that still holds the previous call's partial sums.
+an allocation).  It must give what the context-based entry point gives, call after call, and take no
+device memory after the first one.
 
 Collected last on purpose: a run that stops at the first failure has then run every other test.
 """
@@ -26,7 +26,7 @@ def test_noalloc_gemm_matches_context_gemm_twice_in_a_row():
             w = wl.normal_tensor(21 + call, 2, (n, k), 0.05, device="cuda", dtype=torch.bfloat16)
             out = torch.full((rows, n), float("nan"), dtype=torch.float32, device="cuda")
             if call == 0:
-                # the first call on a device looks up the array (and may make the driver load the kernels' module):
+                # the first call on a device maps the error words (and may make the driver load the kernels' module):
                 # allowed to take device memory once, before the calls that must not
                 assert b.gemm_bf16_noalloc(x, w, out, split) == 0
                 out.fill_(float("nan"))
@@ -61,7 +61,7 @@ def test_noalloc_gemm_rejects_what_does_not_fit():
     x = torch.zeros((256, 64), dtype=torch.bfloat16, device="cuda")
     w = torch.zeros((4096, 64), dtype=torch.bfloat16, device="cuda")
     out = torch.zeros((256, 4096), dtype=torch.float32, device="cuda")
-    assert b.gemm_bf16_noalloc(x, w, out, 1) == -5           # 256*4096 floats exceed the 4 MiB array: SSD_ERR_OVERFLOW
+    assert b.gemm_bf16_noalloc(x, w, out, 1) == -5           # 256*4096 floats exceed the interface's limit: SSD_ERR_OVERFLOW
     assert b.gemm_bf16_noalloc(x[:128], w, out[:128], 1) == 0
     assert b.gemm_bf16_noalloc(x[:128], w, out[:128], 3) == -5
     assert b.gemm_bf16_noalloc(x[:128], w, out[:128], 9) == -2  # split_k outside [1, 8]: SSD_ERR_SHAPE
