@@ -205,7 +205,7 @@ attn_fill_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
     asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kRegsOther));
     if (warp == 9) {
       // ------------------------------------------------------------------ copies
-      if (lane == 0) {
+      if (elect_one()) {
         mbar_expect_tx(bar_q, (uint32_t)(kQ * kTileBytes));
         for (int i = 0; i < kQ; ++i)
           for (int half = 0; half < 2; ++half)
@@ -242,9 +242,10 @@ attn_fill_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
       const uint32_t idesc_pv = idesc | (1u << 16);                // B is MN-major: V as stored
       // (the address field of a descriptor counts 16-byte units)
       const uint64_t qdesc = make_desc(smem_u32(sQ), 16, 1024), kdesc = make_desc(smem_u32(sK), 16, 1024), vdesc = make_desc(smem_u32(sV), kHalfBytes, 1024);
-      auto issue_s = [&](int i, int j) {
-        const uint64_t qd = qdesc + (uint32_t)(i * (kTileBytes >> 4)), kd = kdesc + (uint32_t)((j % kStages) * (kTileBytes >> 4));
-        if (elect_one()) {
+      // (one lane, elected once, walks the loop: an election in each step costs more than the MMAs' issue)
+      if (elect_one()) {
+        auto issue_s = [&](int i, int j) {
+          const uint64_t qd = qdesc + (uint32_t)(i * (kTileBytes >> 4)), kd = kdesc + (uint32_t)((j % kStages) * (kTileBytes >> 4));
 #pragma unroll
           for (int k = 0; k < 8; ++k) {
             const uint32_t off = (uint32_t)((k >> 2) * kHalfBytes + (k & 3) * 32) >> 4;
@@ -252,45 +253,45 @@ attn_fill_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
           }
           tc_commit(bar_s + 8 * i);
           if (i == kQ - 1) tc_commit(bar_ke + 8 * (j % kStages));
-        }
-        __syncwarp();
-      };
-      auto issue_pv = [&](int i, int j, int half) {              // keys [64 half, +64) of the tile
-        const uint64_t vd = vdesc + (uint32_t)((j % kStages) * (kTileBytes >> 4));
-        if (elect_one()) {
+        };
+        auto issue_pv = [&](int i, int j, int half) {              // keys [64 half, +64) of the tile
+          const uint64_t vd = vdesc + (uint32_t)((j % kStages) * (kTileBytes >> 4));
 #pragma unroll
-          for (int k = 4 * half; k < 4 * half + 4; ++k)
-            tc_mma_ts(tmem_base + 128u * (kQ + i), tmem_base + 128u * i + 8u * k, vd + (uint32_t)(2 * k * 64), idesc_pv, (uint32_t)((j | k) != 0));
+          for (int k = 0; k < 4; ++k)
+            tc_mma_ts(tmem_base + 128u * (kQ + i), tmem_base + 128u * i + 8u * (4 * half + k), vd + (uint32_t)(2 * (4 * half + k) * 64), idesc_pv,
+                      (uint32_t)((j | half | k) != 0));
           if (half == 1 && i == kQ - 1) tc_commit(bar_ve + 8 * (j % kStages));
           if (half == 1 && j == n_kt - 1) tc_commit(bar_o + 8 * i);
-        }
-        __syncwarp();
-      };
-      auto wait = [&](uint32_t bar, uint32_t parity) -> bool { return __all_sync(0xffffffffu, mbar_wait(bar, parity, abort_flag) ? 1 : 0) != 0; };
-      ok = wait(bar_q, 0) && wait(bar_kf, 0);
-      tc_fence_after();
-      if (ok)
-        for (int i = 0; i < kQ; ++i) issue_s(i, 0);
-      for (int j = 0; j < n_kt && ok; ++j) {
-        ok = wait(bar_vf + 8 * (j % kStages), (uint32_t)((j / kStages) & 1));
-        for (int i = 0; i < kQ && ok; ++i) {
-          for (int half = 0; half < 2 && ok; ++half) {
-            ok = wait(bar_p + 16 * i + 8 * half, (uint32_t)(j & 1));
-            if (!ok) break;
-            tc_fence_after();
-            issue_pv(i, j, half);
-          }
-          if (!ok) break;
-          if (j + 1 < n_kt) {
-            if (i == 0) {
-              ok = wait(bar_kf + 8 * ((j + 1) % kStages), (uint32_t)(((j + 1) / kStages) & 1));
+        };
+        auto wait = [&](uint32_t bar, uint32_t parity) -> bool { return mbar_wait(bar, parity, abort_flag); };
+        ok = wait(bar_q, 0) && wait(bar_kf, 0);
+        tc_fence_after();
+        if (ok)
+          for (int i = 0; i < kQ; ++i) issue_s(i, 0);
+        for (int j = 0; j < n_kt && ok; ++j) {
+          ok = wait(bar_vf + 8 * (j % kStages), (uint32_t)((j / kStages) & 1));
+#pragma unroll
+          for (int i = 0; i < kQ; ++i) {
+#pragma unroll
+            for (int half = 0; half < 2; ++half) {
+              if (ok) ok = wait(bar_p + 16 * i + 8 * half, (uint32_t)(j & 1));
               if (!ok) break;
               tc_fence_after();
+              issue_pv(i, j, half);
             }
-            issue_s(i, j + 1);             // (in order behind O += P V, which still reads P from the same columns)
+            if (!ok) break;
+            if (j + 1 < n_kt) {
+              if (i == 0) {
+                ok = wait(bar_kf + 8 * ((j + 1) % kStages), (uint32_t)(((j + 1) / kStages) & 1));
+                if (!ok) break;
+                tc_fence_after();
+              }
+              issue_s(i, j + 1);             // (in order behind O += P V, which still reads P from the same columns)
+            }
           }
         }
       }
+      __syncwarp();
     }
   } else if ((warp >> 2) < kQ) {
     asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(kRegsSoftmax));

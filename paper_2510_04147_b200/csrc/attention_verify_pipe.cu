@@ -295,40 +295,38 @@ attn_verify_pipe_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
     // (the address field of a descriptor counts 16-byte units)
     const uint64_t qdesc = make_desc(smem_u32(sQ), 16, 1024), kdesc = make_desc(smem_u32(sKs), 16, 1024);
     const uint64_t pdesc = make_desc(smem_u32(sP), 16, 1024), vdesc = make_desc(smem_u32(sVs), kHalfBytes, 1024);
-    auto issue_s = [&](int u) {                        // S[u & 1] = Q . K(u)^T: eight k16 steps over the head dimension
-      const uint64_t kd = kdesc + (uint32_t)((u % kStagesK) * (kTileBytes >> 4));
-      if (elect_one()) {
+    // One lane, elected once, walks the loop: an election and a vote in each step cost a few hundred clocks of every tile's chain.
+    if (elect_one()) {
+      auto issue_s = [&](int u) {                      // S[u & 1] = Q . K(u)^T: eight k16 steps over the head dimension
+        const uint64_t kd = kdesc + (uint32_t)((u % kStagesK) * (kTileBytes >> 4));
 #pragma unroll
         for (int k = 0; k < 8; ++k) {
           const uint32_t off = (uint32_t)((k >> 2) * kHalfBytes + (k & 3) * 32) >> 4;
           tc_mma_bf16(tmem_base + (uint32_t)(u & 1) * 128u, qdesc + off, kd + off, idesc, (uint32_t)(k != 0));
         }
         tc_commit(bar_s0 + 8u * (uint32_t)(u & 1));
+      };
+      auto wait = [&](uint32_t bar, uint32_t parity) -> bool { return mbar_wait(bar, parity, abort_flag); };
+      ok = wait(bar_q, 0) && wait(bar_k0, 0);
+      if (ok) {
+        tc_fence_after();
+        issue_s(0);
       }
-      __syncwarp();
-    };
-    auto wait = [&](uint32_t bar, uint32_t parity) -> bool { return __all_sync(0xffffffffu, mbar_wait(bar, parity, abort_flag) ? 1 : 0) != 0; };
-    ok = wait(bar_q, 0) && wait(bar_k0, 0);
-    if (ok) {
-      tc_fence_after();
-      issue_s(0);
-    }
 #pragma unroll 1
-    for (int u = 0; u < n_tiles && ok; ++u) {
-      if (u + 1 < n_tiles) {
-        ok = wait(bar_k0 + 8u * (uint32_t)((u + 1) & 1), (uint32_t)(((u + 1) >> 1) & 1));
-        if (ok && u >= 1) ok = wait(bar_sfree0 + 8u * (uint32_t)((u - 1) & 1), (uint32_t)(((u - 1) >> 1) & 1));
+      for (int u = 0; u < n_tiles && ok; ++u) {
+        if (u + 1 < n_tiles) {
+          ok = wait(bar_k0 + 8u * (uint32_t)((u + 1) & 1), (uint32_t)(((u + 1) >> 1) & 1));
+          if (ok && u >= 1) ok = wait(bar_sfree0 + 8u * (uint32_t)((u - 1) & 1), (uint32_t)(((u - 1) >> 1) & 1));
+          if (!ok) break;
+          tc_fence_after();
+          issue_s(u + 1);
+        }
+        ok = wait(bar_p, (uint32_t)(u & 1)) && wait(bar_v0 + 8u * (uint32_t)(u & 1), (uint32_t)((u >> 1) & 1));
         if (!ok) break;
         tc_fence_after();
-        issue_s(u + 1);
-      }
-      ok = wait(bar_p, (uint32_t)(u & 1)) && wait(bar_v0 + 8u * (uint32_t)(u & 1), (uint32_t)((u >> 1) & 1));
-      if (!ok) break;
-      tc_fence_after();
-      // O (+)= P . V: eight k16 steps over the keys.  P is K-major (keys contiguous); V is used as stored,
-      // [key][hd] = MN-major: 8-key groups 1024 B apart, the two 64-column halves 16 KB apart.
-      const uint64_t vd = vdesc + (uint32_t)((u % kStagesV) * (kTileBytes >> 4));
-      if (elect_one()) {
+        // O (+)= P . V: eight k16 steps over the keys.  P is K-major (keys contiguous); V is used as stored,
+        // [key][hd] = MN-major: 8-key groups 1024 B apart, the two 64-column halves 16 KB apart.
+        const uint64_t vd = vdesc + (uint32_t)((u % kStagesV) * (kTileBytes >> 4));
 #pragma unroll
         for (int k = 0; k < 8; ++k) {
           if (kTmemP) tc_mma_bf16_ta(tmem_O, tmem_P + (uint32_t)(u & 1) * 64u + 8u * k, vd + (uint32_t)(2 * k * 64), idesc_pv, (uint32_t)((u | k) != 0));
@@ -336,12 +334,12 @@ attn_verify_pipe_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
         }
         tc_commit(bar_o0 + 8u * (uint32_t)(u & 1));
       }
-      __syncwarp();
+      if (!ok) raise_word(a.err_flag, 6);
     }
-    if (!ok && lane == 0) raise_word(a.err_flag, 6);
+    __syncwarp();
   } else if (warp > kPipeThreads / 32) {
     // ================================================================== copy warp
-    if (lane == 0) {
+    if (elect_one()) {
       // The cache is not written below the rows' own positions by any kernel of this forward, so cached tiles may be
       // requested before the dependency wait - unless the slot -> sequence map is only known on the device.
       const bool early = a.map.n_inline > 0 || a.map.seq_map == nullptr;

@@ -281,7 +281,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ 
   bool epi_ok = false;       // epilogue threads: the accumulator is complete
   if (warp == 0) {
     // ------------------------------------------------------------------ TMA producer
-    if (lane == 0) {
+    if (elect_one()) {
       const uint32_t stage_bytes = (uint32_t)(kWTileBytes + x_tile_bytes);
       int issued = 0;
       bool ok = true;
@@ -347,9 +347,9 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ 
     }
   } else if (warp == 1) {
     // ------------------------------------------------------------------ MMA issuer
-    // The whole warp walks the loop and one elected lane issues: with warp-uniform addresses and descriptors an MMA is a
-    // few instructions.
-    if (leader) {        // (in a pair the even CTA issues for both)
+    // One lane, elected once, walks the whole loop: with warp-uniform addresses and descriptors an MMA is a few instructions, and
+    // four of them, a commit and a wait take 250 clocks; with an election in each turn 350 (a pair 530).
+    if (leader && elect_one()) {        // (in a pair the even CTA issues for both)
       // M = 128 features of this CTA, or 256 = the pair's two weight tiles; N = the padded rows
       const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(p.npad >> 3) << 17) |
                              ((uint32_t)((ts ? 2 * kTileM : kTileM) >> 4) << 24);
@@ -360,33 +360,29 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ 
       uint32_t phase = 0;
       for (int it = 0; it < n_kb; ++it) {
         ok = mbar_wait(full0 + 8 * s, phase, abort_flag, p.wait_limit_ns);
-        ok = __all_sync(0xffffffffu, ok);
         if (!ok) break;
         tc_fence_after();
         // (the address field of a descriptor counts 16-byte units: a stage and a k16 step are additions)
         const uint64_t wd = wdesc0 + (uint32_t)(s * (kWTileBytes >> 4)), xd = xdesc0 + (uint32_t)(s * (x_tile_bytes >> 4));
-        if (elect_one()) {
 #pragma unroll
-          for (int k = 0; k < kBlockK / 16; ++k) {
-            if constexpr (ts) tc_mma_bf16_pair(tmem_base, wd + 2 * k, xd + 2 * k, idesc, (uint32_t)((it | k) != 0));
-            else tc_mma_bf16(tmem_base, wd + 2 * k, xd + 2 * k, idesc, (uint32_t)((it | k) != 0));
-          }
-          // a pair's commits arrive on both CTAs' barriers; only stages that will be refilled need one
-          if constexpr (!ts) tc_commit(empty0 + 8 * s);
-          else if (it + p.stages < n_kb) tc_commit_pair(empty0 + 8 * s);
-          if (it + 1 == n_kb) {
-            if constexpr (ts) tc_commit_pair(smem_addr(acc_bar));
-            else tc_commit(smem_addr(acc_bar));
-          }
+        for (int k = 0; k < kBlockK / 16; ++k) {
+          if constexpr (ts) tc_mma_bf16_pair(tmem_base, wd + 2 * k, xd + 2 * k, idesc, (uint32_t)((it | k) != 0));
+          else tc_mma_bf16(tmem_base, wd + 2 * k, xd + 2 * k, idesc, (uint32_t)((it | k) != 0));
         }
-        __syncwarp();
+        // a pair's commits arrive on both CTAs' barriers; only stages that will be refilled need one
+        if constexpr (!ts) tc_commit(empty0 + 8 * s);
+        else if (it + p.stages < n_kb) tc_commit_pair(empty0 + 8 * s);
         if (++s == p.stages) { s = 0; phase ^= 1u; }
       }
-      if (!ok && lane == 0) {
+      if (ok) {
+        if constexpr (ts) tc_commit_pair(smem_addr(acc_bar));
+        else tc_commit(smem_addr(acc_bar));
+      } else {
         *abort_flag = 1;
         raise_word(p.err_flag, 2);
       }
     }
+    __syncwarp();
   } else {
     // ------------------------------------------------------------------ epilogue
     const int quad = warp & 3;                 // TMEM lane quadrant this warp may read

@@ -261,7 +261,7 @@ gemm_dense_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant
 
   if (warp == 0) {
     // ------------------------------------------------------------------ TMA producer
-    if (lane == 0) {
+    if (elect_one()) {
       // (one thread issues everything: what it computes per K block is what bounds a stage, so positions run along and
       // nothing is divided in the loop)
       const int my_tiles = (total - pair + n_pairs - 1) / n_pairs;
@@ -320,9 +320,9 @@ gemm_dense_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant
     }
   } else if (warp == 1) {
     // ------------------------------------------------------------------ MMA issuer (the even CTA, for both)
-    // The whole warp walks the loop and one elected lane issues: with warp-uniform addresses and descriptors an MMA is a
-    // few instructions (from one lane's registers each took 70 clocks to issue, 580 per K block in all).
-    if (leader) {
+    // One lane, elected once, walks the whole loop: with warp-uniform addresses and descriptors an MMA is a few instructions
+    // (from a diverged lane's registers each took 70 clocks to issue, 580 per K block in all).
+    if (leader && elect_one()) {
       const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(kFeat >> 3) << 17) | ((uint32_t)(kTileRows >> 4) << 24);
       bool ok = true;
       const uint32_t full0 = smem_addr(full_bar), empty0 = smem_addr(empty_bar);
@@ -334,7 +334,6 @@ gemm_dense_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant
           const int buf = nth % kBufs;
           if (nth >= kBufs) {
             ok = mbar_wait(smem_addr(&acc_empty[buf]), (uint32_t)((nth / kBufs) & 1) ^ 1u, abort_flag, p.wait_limit_ns);
-            ok = __all_sync(0xffffffffu, ok);
             if (!ok) break;
             tc_fence_after();
           }
@@ -342,23 +341,20 @@ gemm_dense_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant
           const int kb0 = split * n_kb / p.splits, kb1 = (split + 1) * n_kb / p.splits;
           for (int kb = kb0; kb < kb1; ++kb) {
             ok = mbar_wait(full0 + 8 * s, phase, abort_flag, p.wait_limit_ns);
-            ok = __all_sync(0xffffffffu, ok);
             if (!ok) break;
             // (the address field of a descriptor counts 16-byte units: a stage and a k16 step are additions)
             const uint64_t xd = xdesc0 + (uint32_t)(s * (kStageBytes >> 4)), wd = wdesc0 + (uint32_t)(s * (kStageBytes >> 4));
-            if (elect_one()) {
 #pragma unroll
-              for (int k = 0; k < kBlockK / 16; ++k) tc_mma_bf16_pair(tmem_d, xd + 2 * k, wd + 2 * k, idesc, (uint32_t)(((kb - kb0) | k) != 0));
-              tc_commit_pair(empty0 + 8 * s);
-              if (kb + 1 == kb1) tc_commit_pair(smem_addr(&acc_full[buf]));
-            }
-            __syncwarp();
+            for (int k = 0; k < kBlockK / 16; ++k) tc_mma_bf16_pair(tmem_d, xd + 2 * k, wd + 2 * k, idesc, (uint32_t)(((kb - kb0) | k) != 0));
+            tc_commit_pair(empty0 + 8 * s);
             if (++s == kStages) { s = 0; phase ^= 1u; }
           }
+          if (ok) tc_commit_pair(smem_addr(&acc_full[buf]));
         }
       }
-      if (!ok && lane == 0) { *abort_flag = 1; raise_word(p.err_flag, 2); }
+      if (!ok) { *abort_flag = 1; raise_word(p.err_flag, 2); }
     }
+    __syncwarp();
   } else {
     // ------------------------------------------------------------------ epilogue
     const int quad = warp & 3, group = (warp - 2) >> 2;
