@@ -114,7 +114,7 @@ struct ssd_ctx {
 
   int split_qkv = 1, split_o = 1, split_down = 1, kv_split_opt = 0;
   int two_sm_rows = 128;                   // projections pair their tiles (two-SM MMA) from this many rows on; 0 = never
-  int dense_rows = 240;          // forwards of more rows may take the dense projection kernel
+  int dense_rows = 240;          // forwards of more rows may take the dense projection kernel, of more than two thirds of it the evenly shared one
   int attn_impl = 1;                       // 1: tcgen05 attention where the shape allows; 0: mma.sync form only
   int64_t launches = 0;
   int gemm_max_stages = 0;       // tuning: cap on the projection kernel's ring depth (0: none)
@@ -364,6 +364,15 @@ int run_gemm_dense(ssd_ctx* c, GemmArgs g, int sub) {
   return SSD_OK;
 }
 
+int run_gemm_wave(ssd_ctx* c, GemmArgs g, int sub) {
+  Scope sc(c, SSD_PROF_GEMM, (double)g.N * g.K * 2.0, 1, sub);
+  g.err_flag = c->flags;
+  g.wait_limit_ns = (unsigned long long)c->wait_limit_us * 1000ull;
+  const int rc = launch_gemm_wave(c->st, g);
+  if (rc != 0) return fail(c, rc, "evenly shared projection kernel rejected R=%d N=%d K=%d epi=%d (code %d)", g.R, g.N, g.K, g.epi, rc);
+  return SSD_OK;
+}
+
 bool all_loaded(const ssd_ctx* c) {
   if (c->loaded_globals != 7u) return false;
   for (const LayerW& l : c->L)
@@ -418,6 +427,13 @@ int forward(ssd_ctx* c, int kind, const int* ids_dev, int R, RowMap map, int n_s
   const bool may = R > c->dense_rows;
   const bool dense_gu = may && (R <= 256 || R * 16 >= (R + 255) / 256 * 256 * 13);
   const bool dense_qkv = may && (R > 384 || (R <= 256 && gemm_tiles(c->nqkv) >= 74));
+  // Of 161 to 256 rows, q|k|v and gate|up share their features out evenly (where that is less than the turns of whole tiles).  us of
+  // eight layers with the LM head, neither / q|k|v / gate|up, d 4096, ffn 12288 (96 and 192 tiles): 128 rows 1241 / 1251 / 1262,
+  // 160 1420 / 1410 / 1422, 192 1545 / 1533 / 1499, 224 1742 / 1692 / 1660, 256 1766 / 1696 / 1705; d 3584, ffn 18944 (36 tiles of
+  // four splits; 296 tiles go evenly as they are): 128 rows 1307 / 1300 / 1343, 192 1596 / 1575 / 1613, 256 1773 / 1738 / 1783.
+  const bool even = R <= 256 && 3 * R > 2 * c->dense_rows;
+  const bool even_qkv = even && hd == 128 && gemm_wave_fits(c->nqkv, R, c->split_qkv);
+  const bool even_gu = even && gemm_wave_fits(2 * c->ffn_pad, R, 1) && gemm_wave_gains(2 * c->ffn_pad);
   const bool dense_o = may && R > 256, dense_down = may && R > 448;
   // The attention takes finished (rotated, bf16) q, k and v: the tcgen05 form, and the cache-fill forward, whose K/V go to
   // the cache.  (A function of the node width, never of the number of nodes.)
@@ -463,7 +479,10 @@ int forward(ssd_ctx* c, int kind, const int* ids_dev, int R, RowMap map, int n_s
       o.map = map;
     }
     int rc;
-    if (dense_qkv && bf16_qkv) {
+    if (even_qkv && bf16_qkv) {
+      g.epi = EPI_QKV; g.qkv = &o;
+      rc = run_gemm_wave(c, g, SSD_PROF_GEMM_QKV);
+    } else if (dense_qkv && bf16_qkv) {
       g.epi = EPI_QKV; g.qkv = &o;         // rotary embedding, rounding and the cache rows in the projection's epilogue
       rc = run_gemm_dense(c, g, SSD_PROF_GEMM_QKV);
     } else {
@@ -530,7 +549,7 @@ int forward(ssd_ctx* c, int kind, const int* ids_dev, int R, RowMap map, int n_s
     g.splits = 1;
     g.epi = EPI_SWIGLU; g.act = c->act; g.act_pitch = c->ffn_pad;
     consume_norm(g);
-    rc = dense_gu ? run_gemm_dense(c, g, SSD_PROF_GEMM_GU) : run_gemm(c, g, SSD_PROF_GEMM, SSD_PROF_GEMM_GU);
+    rc = even_gu ? run_gemm_wave(c, g, SSD_PROF_GEMM_GU) : dense_gu ? run_gemm_dense(c, g, SSD_PROF_GEMM_GU) : run_gemm(c, g, SSD_PROF_GEMM, SSD_PROF_GEMM_GU);
     if (rc) return rc;
     // ---- down projection + residual + next norm
     g = GemmArgs{};

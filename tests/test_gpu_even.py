@@ -1,0 +1,46 @@
+"""The evenly shared projections (q|k|v and gate|up of up to 256 rows) against the skinny kernel: the same K ranges in the same
+order, so the bits of a forward are the same.  Row counts around the halves of a CTA pair (8-row steps, quarters of 32 rows, 128),
+units that end inside a weight tile, one and two MMAs to a unit, one and four K splits."""
+import numpy as np
+import pytest
+
+from paper_2510_04147_b200 import workloads as wl
+
+pytestmark = pytest.mark.gpu
+
+BASE = wl.TINY.replace(n_layers=2, vocab=512, head_dim=128, weight_dtype="bf16")
+SHAPES = {
+    # units of 16 couples (the least), most of the last ones missing; K ends inside a K block
+    "narrow": BASE.replace(name="even_narrow", d_model=328, n_heads=4, n_kv_heads=2, d_ffn=200),
+    # four K splits with accumulators of their own; units of 136 and of 256 couples (two MMAs)
+    "splits": BASE.replace(name="even_splits", d_model=1024, n_heads=28, n_kv_heads=4, d_ffn=9664),
+    "wide": BASE.replace(name="even_wide", d_model=512, n_heads=32, n_kv_heads=32, d_ffn=18944),
+}
+
+
+@pytest.mark.parametrize("shape,prompt,block,nodes", [
+    ("narrow", 5, 1, 1), ("narrow", 33, 13, 1), ("narrow", 250, 13, 13), ("narrow", 256, 24, 9),
+    ("splits", 17, 16, 1), ("splits", 255, 23, 11), ("splits", 161, 32, 8),
+    ("wide", 9, 9, 2), ("wide", 129, 24, 7), ("wide", 256, 16, 16),
+])
+def test_even_and_skinny_projections_give_the_same_bits(shape, prompt, block, nodes):
+    from paper_2510_04147_b200 import binding
+    w = SHAPES[shape].replace(prompt_len=prompt, batch=1, block_len=block, gen_len=block)
+    prompts = wl.make_prompts(w).numpy()
+    rng = np.random.default_rng(prompt)
+    ids = rng.integers(0, w.vocab - 1, (1, nodes, block))
+    masked = np.ones(ids.shape, bool)
+    ssd = binding.Ssd(binding.config_from_workload(w, max_drafts=nodes - 1))
+    out = []
+    try:
+        ssd.load_workload_weights(w)
+        for dense_rows in (1 << 20, 0):          # (0: every forward of up to 256 rows)
+            ssd.set_option("dense_rows", dense_rows)
+            ssd.prefill(prompts)
+            caches = [x for l in range(w.n_layers) for x in ssd.read_cache(l, 0, prompt)]
+            out.append(caches + [x for x in ssd.verify_forward(ids, masked, want_logits=True)])
+    finally:
+        ssd.destroy()
+    assert all(np.isfinite(x).all() for x in out[0])
+    for x, y in zip(*out):
+        assert np.array_equal(x, y)
