@@ -20,9 +20,13 @@
 // columns; a tile of 32 or 64 rows is replicated to 128 lanes so that more threads share a row.  The order of the tiles
 // and of every sum is fixed by the shapes alone, so a row's bits do not depend on what shares the forward with it.
 //
-// Few (head, sequence) pairs leave most SMs idle while one CTA walks all tiles: the tiles are then split over the CTAs
-// of a cluster, which push (max, sum, unnormalised output) of a row to its owner through distributed shared memory; the owner
-// merges in part order.
+// Few (head, sequence) pairs leave most SMs idle while one CTA walks all tiles: the tiles are then cut into parts, which the CTAs of
+// a cluster share; they push (max, sum, unnormalised output) of a row to its owner through distributed shared memory, and the
+// owner merges in part order.  With several query tiles a CTA of its own for every part is more CTAs than SMs, in two or three
+// turns: then each CTA has two parts, or all of them, one after the other, and merges them in registers - the same parts and the
+// same operations, so the same bits.  us a layer (live stream), a CTA for every part / now: 512 keys, 32 heads, 160 rows 27.8 /
+// 21.6, 320 rows 45.2 / 28.6; 1024 keys, 28 heads, 192 rows 32.2 / 25.7, 320 rows 51.6 / 36.6; two sequences of 700 keys, 28 heads,
+// 64 rows 17.8 / 11.6.
 //
 // Bound by the serial chain of a tile, not by bytes, except for long prefixes under small query tiles.  Of a 128-row tile's
 // 3400 clocks (clock64 at each step, 4096 keys) the scores' maximum took 580, the wait for O += P V 425, exponentials, sums and P
@@ -52,7 +56,7 @@ constexpr int kHalfBytes = kKeys * 128;     // one 64-column half of a 128-row t
 constexpr int kTileBytes = 2 * kHalfBytes;  // a [128][128] bf16 tile
 constexpr int kStagesK = 2, kStagesV = 2;      // + one P tile
 constexpr int kMergePitch = kHD + 4;           // floats per row of the merge buffer
-constexpr int kMergeRows = 128 + kAttnMaxClusterParts;      // [part][owned rows], rounded up
+constexpr int kMergeRows = 232;                 // [entry][owned rows]: seven entries of 32 at most, rounded up
 constexpr unsigned long long kPipeWaitLimitNs = 2000000000ull;
 
 __device__ __forceinline__ unsigned long long gtimer_ns() {
@@ -216,10 +220,25 @@ __device__ __forceinline__ uint32_t tile_off(int row, int ch) {
 }
 
 // Tiles of one (head, sequence): 0 = node-local, 1 .. n_a = cached keys [0, len_a), n_a + 1 .. = the len_b keys from
-// cache row `row_b` on.  `npt` nodes per query tile, `t_pad` key slots per node in tile 0, `n_parts` CTAs per cluster.
+// cache row `row_b` on.  `npt` nodes per query tile, `t_pad` key slots per node in tile 0.  The tiles are cut into `n_parts` parts with
+// a softmax of their own; a cluster of `n_ctas` CTAs has n_parts / n_ctas consecutive ones each.
 struct PipeShape {
-  int len_a, n_a, len_b, row_b, n_all, npt, t_pad, n_parts;
+  int len_a, n_a, len_b, row_b, n_all, npt, t_pad, n_parts, n_ctas;
+  __host__ __device__ int begin(int part) const { return part * n_all / n_parts; }      // first tile of a part
 };
+
+// Parts are merged one after the other, (((0, 1), 2), 3): sums and outputs of what came before and of the next part, each against
+// the larger of the two maxima.  The same operations whether one thread has met both or they come from two CTAs.
+struct Merge { float m, before, next; };                // new maximum, factors of the two sides
+__device__ __forceinline__ Merge merge_of(float m_before, float m_next) {
+  Merge g;
+  g.m = fmaxf(m_before, m_next);
+  const float use = g.m == -INFINITY ? 0.f : g.m;
+  g.before = ex2(m_before - use);
+  g.next = ex2(m_next - use);
+  return g;
+}
+__device__ __forceinline__ float merged(const Merge& g, float before, float next) { return __fmaf_rn(next, g.next, __fmul_rn(before, g.before)); }
 
 template <int QT>
 __global__ void __launch_bounds__(kPipeBlock, 1)
@@ -245,7 +264,8 @@ attn_verify_pipe_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
 
   pdl_launch_dependents();
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const int part = blockIdx.x % g.n_parts, h = blockIdx.x / g.n_parts;      // the cluster spans x
+  const int rank = blockIdx.x % g.n_ctas, h = blockIdx.x / g.n_ctas;        // the cluster spans x
+  const int per_cta = g.n_parts / g.n_ctas, part0 = rank * per_cta;         // this CTA's parts
   const int rps = a.map.rows_per_seq, T = a.map.T;
   const int tile_rows = g.npt * T;                      // query rows of a tile: whole nodes
   const int q_tiles = (rps + tile_rows - 1) / tile_rows;
@@ -255,7 +275,7 @@ attn_verify_pipe_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
   const size_t grow0 = (size_t)slot * rps + lr0;
   const int rows_here = min(tile_rows, rps - lr0), nodes_here = rows_here / T, node0 = (int)grow0 / T;     // (nodes of all sequences)
   // this CTA's tiles: global tile index first + u, u = 0 .. n_tiles - 1
-  const int first = part * g.n_all / g.n_parts, n_tiles = (part + 1) * g.n_all / g.n_parts - first;
+  const int first = g.begin(part0), n_tiles = g.begin(part0 + per_cta) - first;
 
   if (tid == 0) {
     for (int i = 0; i < 12; ++i) mbar_init(smem_u32(&bars[i]), (i == 5 || i == 8 || i == 9) ? kPipeThreads / 32 : 1);
@@ -312,8 +332,11 @@ attn_verify_pipe_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
         tc_fence_after();
         issue_s(0);
       }
+      int next_part = part0 + 1, fresh_at = 0;             // tile whose O += P V starts a part's output
 #pragma unroll 1
       for (int u = 0; u < n_tiles && ok; ++u) {
+        const bool fresh = u == fresh_at;
+        if (fresh) fresh_at = g.begin(next_part++) - first;
         if (u + 1 < n_tiles) {
           ok = wait(bar_k0 + 8u * (uint32_t)((u + 1) & 1), (uint32_t)(((u + 1) >> 1) & 1));
           if (ok && u >= 1) ok = wait(bar_sfree0 + 8u * (uint32_t)((u - 1) & 1), (uint32_t)(((u - 1) >> 1) & 1));
@@ -329,8 +352,8 @@ attn_verify_pipe_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
         const uint64_t vd = vdesc + (uint32_t)((u % kStagesV) * (kTileBytes >> 4));
 #pragma unroll
         for (int k = 0; k < 8; ++k) {
-          if (kTmemP) tc_mma_bf16_ta(tmem_O, tmem_P + (uint32_t)(u & 1) * 64u + 8u * k, vd + (uint32_t)(2 * k * 64), idesc_pv, (uint32_t)((u | k) != 0));
-          else tc_mma_bf16(tmem_O, pdesc + ((uint32_t)((k >> 2) * kHalfBytes + (k & 3) * 32) >> 4), vd + (uint32_t)(2 * k * 64), idesc_pv, (uint32_t)((u | k) != 0));
+          if (kTmemP) tc_mma_bf16_ta(tmem_O, tmem_P + (uint32_t)(u & 1) * 64u + 8u * k, vd + (uint32_t)(2 * k * 64), idesc_pv, (uint32_t)(!fresh || k != 0));
+          else tc_mma_bf16(tmem_O, pdesc + ((uint32_t)((k >> 2) * kHalfBytes + (k & 3) * 32) >> 4), vd + (uint32_t)(2 * k * 64), idesc_pv, (uint32_t)(!fresh || k != 0));
         }
         tc_commit(bar_o0 + 8u * (uint32_t)(u & 1));
       }
@@ -429,6 +452,25 @@ attn_verify_pipe_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
     const int loc_lo = min(row / T, nodes_here - 1) * g.t_pad;
     const int loc_hi = loc_lo + (a.map.chain_T0 > 0 && lr % T < a.map.chain_T0 ? a.map.chain_T0 : T);   // (finished block: not the next block)
     bool broke = false;                                   // the loop ended at the meeting point, for all threads alike
+    // What the parts before the one in work came to, against their maximum: all of them (this CTA has the first part of all), or the
+    // one before (a CTA further on, whose parts are merged by the rows' owner)
+    float acc[KPT], acc_m = -INFINITY, acc_l = 0.f;
+    bool have = false;
+    auto part_done = [&](float m, float l) {              // the part whose output stands in tensor memory
+      const bool fold = have;
+      const Merge g2 = merge_of(acc_m, m);
+#pragma unroll
+      for (int ch = 0; ch < NCH; ++ch) {
+        float v[16];
+        tmem_ld16(tmem_O + lane_addr + col0 + ch * 16, v);
+#pragma unroll
+        for (int j = 0; j < 16; ++j) acc[ch * 16 + j] = fold ? merged(g2, acc[ch * 16 + j], v[j]) : v[j];
+      }
+      acc_l = fold ? merged(g2, acc_l, l) : l;
+      acc_m = fold ? g2.m : m;
+      have = true;
+    };
+    int next_part = part0 + 1, fresh_at = g.begin(next_part) - first;
     float corr_prev = 1.f;                                // rescale factor of the tile whose sum is still to be added
     auto tile_sum = [&](int u) -> float {                 // the row's sum over tile u, from the eight chunk sums
       const float* q = sSum + (u & 1) * 8 * 128 + row;
@@ -486,6 +528,15 @@ attn_verify_pipe_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
       if (u > 0) {                                          // (every chunk sum of the previous tile is visible now)
         l_row = l_row * corr_prev + tile_sum(u - 1);
       }
+      if (u == fresh_at && u < n_tiles) {                   // this tile starts a part: put the one before away
+        fresh_at = g.begin(++next_part) - first;
+        ok = mbar_wait(bar_o0 + 8u * (uint32_t)((u - 1) & 1), (uint32_t)(((u - 1) >> 1) & 1), abort_flag);
+        tc_fence_after();
+        ok = __all_sync(0xffffffffu, ok ? 1 : 0) != 0;
+        if (ok) part_done(m_row, l_row);
+        m_row = -INFINITY;
+        l_row = 0.f;
+      }
       float m_tile = -INFINITY;
 #pragma unroll
       for (int k = 0; k < REP; ++k) m_tile = fmaxf(m_tile, fmaxf(sMaxU[k * 128 + row], sMaxU[(4 + k) * 128 + row]));
@@ -494,7 +545,7 @@ attn_verify_pipe_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
       const float corr = ex2(m_row - m_use);                // 0 while no visible key has been met
       // the output so far was accumulated against the old maximum: rescale this thread's columns of its lane - unless
       // no row of the warp moved its maximum (a factor of exactly 1 changes nothing)
-      const bool rescale = u > 0 && __any_sync(0xffffffffu, corr != 1.f);
+      const bool rescale = u > 0 && __any_sync(0xffffffffu, corr != 1.f && m_row != -INFINITY);
       // O += P V that must be complete: the previous tile's if the output is rescaled or its P rewritten, else (P in
       // tensor memory, where tiles alternate) the one before
       const int must = (rescale || !kTmemP) ? u - 1 : u - 2;
@@ -571,51 +622,53 @@ attn_verify_pipe_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
       tc_fence_after();
     }
     ok = __all_sync(0xffffffffu, ok ? 1 : 0) != 0;
-    if (ok && g.n_parts == 1) {
+    // this CTA's last part; a CTA that has not the first part of all hands two parts on as two entries
+    const bool two = have && rank > 0;
+    if (ok && !two) part_done(m_row, l_row);
+    if (ok && g.n_ctas == 1) {
       // every copy of a row holds the same O row: a thread normalises and stores the columns it owns, [col0, +KPT)
-      const float inv = 1.f / l_row;
+      const float inv = 1.f / acc_l;
       bf16* dst = a.out + ((grow0 + row) * a.H + h) * kHD + col0;
+      if (row_live) {
 #pragma unroll
-      for (int ch = 0; ch < NCH; ++ch) {
-        float v[16];
-        tmem_ld16(tmem_O + lane_addr + col0 + ch * 16, v);
-        if (row_live) {
-          *reinterpret_cast<uint4*>(dst + ch * 16) =
-              make_uint4(pack_bf16(v[0] * inv, v[1] * inv), pack_bf16(v[2] * inv, v[3] * inv), pack_bf16(v[4] * inv, v[5] * inv),
-                         pack_bf16(v[6] * inv, v[7] * inv));
-          *reinterpret_cast<uint4*>(dst + ch * 16 + 8) =
-              make_uint4(pack_bf16(v[8] * inv, v[9] * inv), pack_bf16(v[10] * inv, v[11] * inv), pack_bf16(v[12] * inv, v[13] * inv),
-                         pack_bf16(v[14] * inv, v[15] * inv));
-        }
-        __syncwarp();
+        for (int j = 0; j < KPT; j += 8)
+          *reinterpret_cast<uint4*>(dst + j) = make_uint4(pack_bf16(acc[j] * inv, acc[j + 1] * inv), pack_bf16(acc[j + 2] * inv, acc[j + 3] * inv),
+                                                          pack_bf16(acc[j + 4] * inv, acc[j + 5] * inv), pack_bf16(acc[j + 6] * inv, acc[j + 7] * inv));
       }
-    } else if (g.n_parts > 1) {
+    } else if (g.n_ctas > 1) {
       // Rows go to their owner, CTA row / rows_per_owner of the cluster: (max, sum) and the unnormalised output, straight
-      // from registers into its shared memory, [part][owned row].  The first cluster barrier says that every CTA is done
+      // from registers into its shared memory, [entry][owned row].  The first cluster barrier says that every CTA is done
       // with its tiles, the second that all rows have arrived; nothing is read remotely, so nobody waits to leave.
       __syncwarp();
       cluster_arrive();
-      const int rpo = (QT + g.n_parts - 1) / g.n_parts, owner = row / rpo, slot_row = part * rpo + row - owner * rpo;
-      const uint32_t dst = map_to_rank(smem + ((size_t)slot_row * kMergePitch + col0) * sizeof(float), (uint32_t)owner);
+      const int rpo = (QT + g.n_ctas - 1) / g.n_ctas, owner = row / rpo, entry = rank == 0 ? 0 : 1 + (rank - 1) * per_cta;
+      const int slot_row = entry * rpo + row - owner * rpo;
+      uint32_t dst = map_to_rank(smem + ((size_t)slot_row * kMergePitch + col0) * sizeof(float), (uint32_t)owner);
       const uint32_t dst_ml = map_to_rank(smem + (size_t)kMergeRows * kMergePitch * sizeof(float) + slot_row * sizeof(float2), (uint32_t)owner);
-      float v[NCH][16];
-      if (ok) {
-#pragma unroll
-        for (int ch = 0; ch < NCH; ++ch) tmem_ld16(tmem_O + lane_addr + col0 + ch * 16, v[ch]);
-      }
       cluster_wait();
       if (ok && row_live) {
 #pragma unroll
-        for (int ch = 0; ch < NCH; ++ch)
+        for (int j = 0; j < KPT; j += 4) st_cluster_f32x4(dst + (uint32_t)j * 4u, acc[j], acc[j + 1], acc[j + 2], acc[j + 3]);
+        if (cw == 0 && hw == 0) st_cluster_f32x2(dst_ml, acc_m, acc_l);
+      }
+      if (ok && two) {
+        dst += (uint32_t)(rpo * kMergePitch * sizeof(float));
 #pragma unroll
-          for (int j = 0; j < 16; j += 4)
-            st_cluster_f32x4(dst + (uint32_t)(ch * 16 + j) * 4u, v[ch][j], v[ch][j + 1], v[ch][j + 2], v[ch][j + 3]);
-        if (cw == 0 && hw == 0) st_cluster_f32x2(dst_ml, m_row, l_row);
+        for (int ch = 0; ch < NCH; ++ch) {
+          float v[16];
+          tmem_ld16(tmem_O + lane_addr + col0 + ch * 16, v);
+          if (row_live) {
+#pragma unroll
+            for (int j = 0; j < 16; j += 4) st_cluster_f32x4(dst + (uint32_t)(ch * 16 + j) * 4u, v[j], v[j + 1], v[j + 2], v[j + 3]);
+          }
+          __syncwarp();
+        }
+        if (row_live && cw == 0 && hw == 0) st_cluster_f32x2(dst_ml + (uint32_t)(rpo * sizeof(float2)), m_row, l_row);
       }
     }
     if (!ok && lane == 0) raise_word(a.err_flag, 6);
   }
-  if (warp >= kPipeThreads / 32 && g.n_parts > 1) {        // (the first cluster barrier, of the threads that push nothing)
+  if (warp >= kPipeThreads / 32 && g.n_ctas > 1) {        // (the first cluster barrier, of the threads that push nothing)
     __syncwarp();
     cluster_arrive();
     cluster_wait();
@@ -625,43 +678,44 @@ attn_verify_pipe_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
   if (warp == kPipeThreads / 32) {
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"(512u) : "memory");
   }
-  if (g.n_parts == 1) return;
+  if (g.n_ctas == 1) return;
   __syncwarp();
   cluster_arrive();
   cluster_wait();
-  // ---- merge: this CTA's rows, the parts added in part order.  (After an error the rows are garbage and the error word is up.)
+  // ---- merge: this CTA's rows, the entries in part order.  (After an error the rows are garbage and the error word is up.)
   if (warp < kPipeThreads / 32) {
-    const int rpo = (QT + g.n_parts - 1) / g.n_parts, r_end = min(rpo, rows_here - part * rpo);
+    const int rpo = (QT + g.n_ctas - 1) / g.n_ctas, r_end = min(rpo, rows_here - rank * rpo), entries = 1 + (g.n_ctas - 1) * per_cta;
     const float* sO = reinterpret_cast<const float*>(smem);
     const float2* sML = reinterpret_cast<const float2*>(sO + kMergeRows * kMergePitch);
     constexpr int TPR = kHD / 8;                            // threads per row, eight columns each
     const int col = (tid % TPR) * 8;
     for (int r = tid / TPR; r < r_end; r += kPipeThreads / TPR) {
-      float M = -INFINITY;
-      for (int pp = 0; pp < g.n_parts; ++pp) M = fmaxf(M, sML[pp * rpo + r].x);
-      float L = 0.f;
-      float4 acc0 = make_float4(0.f, 0.f, 0.f, 0.f), acc1 = acc0;
-      for (int pp = 0; pp < g.n_parts; ++pp) {
-        const float2 ml = sML[pp * rpo + r];
-        const float4* o = reinterpret_cast<const float4*>(sO + (size_t)(pp * rpo + r) * kMergePitch + col);
-        const float4 va = o[0], vb = o[1];
-        const float w = ex2(ml.x - M);
-        L += ml.y * w;
-        acc0.x += va.x * w; acc0.y += va.y * w; acc0.z += va.z * w; acc0.w += va.w * w;
-        acc1.x += vb.x * w; acc1.y += vb.y * w; acc1.z += vb.z * w; acc1.w += vb.w * w;
+      float2 ml = sML[r];
+      float m = ml.x, l = ml.y, o[8];
+      const float4* p = reinterpret_cast<const float4*>(sO + (size_t)r * kMergePitch + col);
+      *reinterpret_cast<float4*>(o) = p[0];
+      *reinterpret_cast<float4*>(o + 4) = p[1];
+      for (int e = 1; e < entries; ++e) {
+        ml = sML[e * rpo + r];
+        p = reinterpret_cast<const float4*>(sO + (size_t)(e * rpo + r) * kMergePitch + col);
+        const float4 va = p[0], vb = p[1];
+        const Merge g2 = merge_of(m, ml.x);
+        o[0] = merged(g2, o[0], va.x); o[1] = merged(g2, o[1], va.y); o[2] = merged(g2, o[2], va.z); o[3] = merged(g2, o[3], va.w);
+        o[4] = merged(g2, o[4], vb.x); o[5] = merged(g2, o[5], vb.y); o[6] = merged(g2, o[6], vb.z); o[7] = merged(g2, o[7], vb.w);
+        l = merged(g2, l, ml.y);
+        m = g2.m;
       }
-      const float inv = 1.f / L;
-      *reinterpret_cast<uint4*>(a.out + ((grow0 + part * rpo + r) * a.H + h) * kHD + col) =
-          make_uint4(pack_bf16(acc0.x * inv, acc0.y * inv), pack_bf16(acc0.z * inv, acc0.w * inv),
-                     pack_bf16(acc1.x * inv, acc1.y * inv), pack_bf16(acc1.z * inv, acc1.w * inv));
+      const float inv = 1.f / l;
+      *reinterpret_cast<uint4*>(a.out + ((grow0 + rank * rpo + r) * a.H + h) * kHD + col) =
+          make_uint4(pack_bf16(o[0] * inv, o[1] * inv), pack_bf16(o[2] * inv, o[3] * inv), pack_bf16(o[4] * inv, o[5] * inv), pack_bf16(o[6] * inv, o[7] * inv));
     }
   }
 }
 
 template <int QT>
-cudaError_t launch_pipe(cudaStream_t st, dim3 grid, size_t smem, int n_parts, const CUtensorMap (&tm)[5], const AttnArgs& a, const PipeShape& g,
+cudaError_t launch_pipe(cudaStream_t st, dim3 grid, size_t smem, const CUtensorMap (&tm)[5], const AttnArgs& a, const PipeShape& g,
                         float scale_log2) {
-  return launch_pdl_cluster(attn_verify_pipe_kernel<QT>, grid, dim3(kPipeBlock), smem, st, (unsigned)n_parts, tm[0], tm[1], tm[2], tm[3], tm[4], a, g,
+  return launch_pdl_cluster(attn_verify_pipe_kernel<QT>, grid, dim3(kPipeBlock), smem, st, (unsigned)g.n_ctas, tm[0], tm[1], tm[2], tm[3], tm[4], a, g,
                             scale_log2);
 }
 
@@ -680,11 +734,22 @@ int launch_attention_verify_pipe(cudaStream_t st, const AttnArgs& a, int n_parts
   g.n_all = 1 + g.n_a + (g.len_b + kKeys - 1) / kKeys;
   g.t_pad = 16;
   while (g.t_pad < T) g.t_pad *= 2;
-  g.n_parts = n_parts < g.n_all ? n_parts : g.n_all;
+  g.n_parts = n_parts < g.n_all ? n_parts : g.n_all;      // (every part has a tile)
   const int qt_rows = rps <= 32 ? 32 : (rps <= 64 ? 64 : 128);
   g.npt = qt_rows / T;
   if (g.npt > kKeys / g.t_pad) g.npt = kKeys / g.t_pad;
   const int q_tiles = (rps + g.npt * T - 1) / (g.npt * T);
+  // How many CTAs share the parts: one for each, one for two, or one for all - the bits are the same.  One CTA to an SM, so many
+  // query tiles take turns if each part has a CTA of its own.  A turn costs some 8 us and 1.5 us a tile, the exchange 3 us, merging
+  // in registers 0.6 us a part (in tenths below; fitted to 1, 2 and 4 CTAs at 5, 9 and 17 tiles).
+  g.n_ctas = g.n_parts;
+  long long best = 0;
+  for (int n : {g.n_parts, g.n_parts / 2, 1}) {
+    if (n < 1 || g.n_parts % n != 0) continue;
+    const long long turns = ((long long)a.H * a.n_seq_slots * q_tiles * n + kSms - 1) / kSms;
+    const long long cost = turns * (80 + 15 * ((g.n_all + n - 1) / n) + (n > 1 ? 30 : 0) + 6 * (g.n_parts / n - 1));
+    if (best == 0 || cost < best) { best = cost; g.n_ctas = n; }
+  }
   const float scale_log2 = (1.0f / sqrtf((float)a.hd)) * 1.4426950408889634f;
   const size_t smem = (size_t)kTileBytes * (2 + kStagesK + kStagesV) + 16384 + 128 + 1024;   // Q, P, K and V stages, softmax exchange
   static bool attr_set[kMaxDevices] = {};        // the shared-memory opt-in is per device
@@ -707,11 +772,11 @@ int launch_attention_verify_pipe(cudaStream_t st, const AttnArgs& a, int n_parts
       encode_tmap_bf16_3d(&tm[3], a.cache_k, kHD, bound, planes, kHD, a.kv_head_stride, kKeys) != 0 ||
       encode_tmap_bf16_3d(&tm[4], a.cache_v, kHD, bound, planes, kHD, a.kv_head_stride, kKeys) != 0)
     return -4;
-  const dim3 grid(a.H * g.n_parts, a.n_seq_slots * q_tiles);
+  const dim3 grid(a.H * g.n_ctas, a.n_seq_slots * q_tiles);
   cudaError_t e;
-  if (qt_rows == 32) e = launch_pipe<32>(st, grid, smem, g.n_parts, tm, a, g, scale_log2);
-  else if (qt_rows == 64) e = launch_pipe<64>(st, grid, smem, g.n_parts, tm, a, g, scale_log2);
-  else e = launch_pipe<128>(st, grid, smem, g.n_parts, tm, a, g, scale_log2);
+  if (qt_rows == 32) e = launch_pipe<32>(st, grid, smem, tm, a, g, scale_log2);
+  else if (qt_rows == 64) e = launch_pipe<64>(st, grid, smem, tm, a, g, scale_log2);
+  else e = launch_pipe<128>(st, grid, smem, tm, a, g, scale_log2);
   return e == cudaSuccess ? 0 : -4;
 }
 

@@ -119,7 +119,7 @@ struct ssd_ctx {
   int64_t launches = 0;
   int gemm_max_stages = 0;       // tuning: cap on the projection kernel's ring depth (0: none)
   int attn_pipe_keys = 1;        // prefixes of at least this many keys take the pipelined attention form (0: never) ...
-  int attn_pipe_ctas = 64;       // ... when the prefilled batch gives it at least this many (head, sequence) CTAs
+  int attn_pipe_ctas = 0;        // ... when the prefilled batch gives it at least this many (head, sequence) CTAs (0: pipe_parts' own line)
   int wait_limit_us = 0;         // bound of the projection kernel's barrier waits (0: the kernel's default, 2 s)
   int starve_gemm_kb = 0;        // test hook for ssd_gemm_bf16: K block (1-based) whose copies are left out
   bool profiling = false;        // mode 1: CUDA events around every launch (serialises the stream)
@@ -211,15 +211,18 @@ int kv_split_for(const ssd_ctx* c, int S) {
   return ks;
 }
 
-// CTAs that share the key tiles of one (query tile, head, sequence) in the tcgen05 attention: one when the prefilled batch
-// gives enough (head, sequence) pairs, else as many as fill the SMs for one sequence.  A function of the heads and the
-// prefilled batch alone - not of the rows or of the sequences still unfinished - so stepwise and SSD forwards of
-// one generation, and a sequence alone and in a batch of the same form, sum in the same order.  With one CTA per SM and
-// clusters inside one of the eight GPCs, four parts are the most that 32 heads find room for at once (five parts of 28 heads
-// took two waves: 20 us where four take 11.5).  One part against four, 512 keys and 32 heads: one sequence 11.4 / 10.4 us at 32
-// rows, 22.9 / 20.4 at 128 (1536 keys: 38.5 / 24.8); two sequences 12.3 / 20.9; eight 28.7 / 74.8.
+// Parts, each with a softmax of its own, that the key tiles of one (query tile, head, sequence) are cut into in the tcgen05
+// attention: one when the prefilled batch gives enough (head, sequence) pairs, else as many as fill the SMs for one sequence.
+// A function of the heads, the keys and the prefilled batch alone - not of the rows or of the sequences still unfinished - so
+// stepwise and SSD forwards of one generation, and a sequence alone and in a batch of the same form, sum in the same order.  (How
+// many CTAs share the parts is the launcher's choice.)  With one CTA per SM and clusters inside one of the eight GPCs, four
+// parts are the most that 32 heads find room for at once (five parts of 28 heads took two waves: 20 us where four take 11.5).
+// One part against four, 32 heads: one sequence of 512 keys 11.4 / 10.4 us at 32 rows; two sequences, where two CTAs share four
+// parts, us of four layers at 64 and 256 rows: 512 keys 607 / 612 and 954 / 952, 1024 keys 625 / 622 and 978 / 964, 2048 keys
+// 662 / 641 and 1045 / 992, 4096 keys 755 / 699 and 1163 / 1042.
 int pipe_parts(const ssd_ctx* c, int S) {
-  if (c->attn_pipe_keys > 0 && S >= c->attn_pipe_keys && c->batch * c->H >= c->attn_pipe_ctas) return 1;
+  const int one_from = c->attn_pipe_ctas > 0 ? c->attn_pipe_ctas : (S >= 1024 ? kSms / 2 + 1 : 64);
+  if (c->attn_pipe_keys > 0 && S >= c->attn_pipe_keys && c->batch * c->H >= one_from) return 1;
   int n = c->kv_split_opt > 0 ? (S + c->kv_split_opt - 1) / c->kv_split_opt + 1 : (c->H <= 16 ? 8 : (c->H <= 32 ? 4 : 2));
   return std::min(std::max(n, 2), kAttnMaxClusterParts);
 }
