@@ -45,6 +45,8 @@ constexpr int kEpiPitch = 132;       // floats per row of the epilogue's transpo
 constexpr int kEpiBufFloats = 32 * kEpiPitch;     // a group's transpose buffer: one chunk
 constexpr unsigned long long kWaitLimitNs = 2000000000ull;   // default bound of a wait, 2 s: far beyond any legitimate one
 
+constexpr int kPairedResidualCtas = 112;         // CTAs in clusters of pairs that all find an SM (14 clusters of eight)
+
 struct TcParams {
   int R, N, K;
   int row_blocks;  // per weight tile
@@ -133,9 +135,9 @@ __device__ __forceinline__ void tma_load_2d_pair(uint32_t dst, const CUtensorMap
       "cp.async.bulk.tensor.2d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4}], [%2];"
       ::"r"(dst), "l"((unsigned long long)map), "r"(bar & kPairLeaderMask), "r"(c0), "r"(c1) : "memory");
 }
-__device__ __forceinline__ void tc_commit_pair(uint32_t bar) {
+__device__ __forceinline__ void tc_commit_pair(uint32_t bar, uint16_t pair_mask) {
   asm volatile("tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;"
-               ::"r"(bar), "h"((uint16_t)3) : "memory");
+               ::"r"(bar), "h"(pair_mask) : "memory");
 }
 __device__ __forceinline__ void tc_mma_bf16_pair(uint32_t tmem_d, uint64_t adesc, uint64_t bdesc, uint32_t idesc,
                                                  uint32_t accumulate) {
@@ -242,8 +244,13 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ 
   const int kb_begin = (int)((long long)split * kb_total / p.splits);
   const int kb_end = (int)((long long)(split + 1) * kb_total / p.splits);
   const int n_kb = kb_end - kb_begin;
-  uint32_t crank = 0u;
-  if constexpr (ts) crank = cluster_ctarank() & 1u;
+  uint32_t crank = 0u;                                          // in the pair
+  uint16_t pair_mask = 3;                                       // the pair among the CTAs of the cluster (EPI_RESIDUAL: a pair for each K split)
+  if constexpr (ts) {
+    const uint32_t r = cluster_ctarank();
+    crank = r & 1u;
+    pair_mask = (uint16_t)(3u << (r & ~1u));
+  }
   const bool leader = crank == 0;
 
   if (threadIdx.x == 0) {
@@ -371,11 +378,11 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ 
         }
         // a pair's commits arrive on both CTAs' barriers; only stages that will be refilled need one
         if constexpr (!ts) tc_commit(empty0 + 8 * s);
-        else if (it + p.stages < n_kb) tc_commit_pair(empty0 + 8 * s);
+        else if (it + p.stages < n_kb) tc_commit_pair(empty0 + 8 * s, pair_mask);
         if (++s == p.stages) { s = 0; phase ^= 1u; }
       }
       if (ok) {
-        if constexpr (ts) tc_commit_pair(smem_addr(acc_bar));
+        if constexpr (ts) tc_commit_pair(smem_addr(acc_bar), pair_mask);
         else tc_commit(smem_addr(acc_bar));
       } else {
         *abort_flag = 1;
@@ -610,7 +617,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ 
     const uint32_t taddr = tmem_base + ((uint32_t)(quad * 32) << 16);
     const int rows_here = min(p.R - row0, p.npad);
     float* scratch = reinterpret_cast<float*>(sW);
-    const int n_ranks = p.splits, rank = (int)cluster_ctarank();
+    const int n_ranks = p.splits, rank = (int)(cluster_ctarank() >> (ts ? 1 : 0));       // one CTA (of this tile) for each split
     const int n_base = tile * kTileM;
     const int f4 = lane * 4;
     const bool resid = p.epi == EPI_RESIDUAL;
@@ -663,7 +670,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ 
 #pragma unroll
           for (int q = 0; q < kQ; ++q) {
             part[u][q] = make_float4(0.f, 0.f, 0.f, 0.f);
-            if (r < limit && q < n_ranks) part[u][q] = ld_cluster_f32x4(map_to_rank(scratch + r * kEpiPitch + f4, (uint32_t)q));
+            if (r < limit && q < n_ranks) part[u][q] = ld_cluster_f32x4(map_to_rank(scratch + r * kEpiPitch + f4, ts ? 2u * (uint32_t)q + crank : (uint32_t)q));
           }
           if (r < limit && col_ok && resid) acc[u] = *reinterpret_cast<const float4*>(p.h + (size_t)(row0 + g0 + r) * p.N + n_base + f4);
         }
@@ -795,7 +802,13 @@ int launch_gemm_tc(cudaStream_t st, const GemmArgs& g) {
   p.w_tiled = g.w_tiled;
   // Pairs of tiles as one two-SM MMA from `two_sm_min_rows` padded rows on (0: never): every SM then takes
   // in half of the activation tile.  The accumulation order is the same, so the row count may decide.
-  p.two_sm = (g.two_sm_min_rows > 0 && p.npad >= g.two_sm_min_rows && g.epi != EPI_RESIDUAL && g.epi != EPI_SUM && (gemm_tiles(g.N) % 2) == 0) ? 1 : 0;
+  // EPI_RESIDUAL: a cluster is then twice as large, and of eight CTAs with an SM each the GPCs have room for 15; so only where that
+  // is enough, or where there are row blocks to take turns anyway.  us in the live stream, without / with: 28 tiles in four
+  // splits, K 18944: 128 rows 30.3 / 29.0, 256 rows 46.0 / 39.8, 320 rows 54.5 / 47.8, 384 rows 72.8 / 58.5; 32 tiles, K 12288: 288
+  // rows 38.8 / 35.5, 384 rows 52.8 / 46.3, but 416 rows 57.2 / 60.3 and 128 rows (16 clusters, two turns) 24.7 / 43.1.
+  const bool pairs_fit = g.epi != EPI_RESIDUAL ||
+                         (2 * g.splits <= kGemmMaxClusterSplits && (gemm_tiles(g.N) * g.splits <= kPairedResidualCtas || (p.row_blocks > 1 && p.npad <= 192)));
+  p.two_sm = (g.two_sm_min_rows > 0 && p.npad >= g.two_sm_min_rows && g.epi != EPI_SUM && pairs_fit && (gemm_tiles(g.N) % 2) == 0) ? 1 : 0;
   uint32_t cols = 32;
   while ((int)cols < p.npad) cols <<= 1;
   p.tmem_cols = cols;
