@@ -191,10 +191,14 @@ int capped_split(int s, int k) {
 // tiles against eight (two CTAs per SM), eight layers: 961 / 964 us at 32 rows, 1062 / 1039 at 64, 1267 / 1253 at 128, 1853 / 1740
 // at 256 (half the reads of the activations, half the partial sums to exchange).
 // A power of two: clusters of five leave so many SMs of a GPC unused that 140 CTAs take two waves (28 tiles: 1019 -> 1164 us).
+// Up to four splits may be down to one K block: the cluster of the splits shares the rows of the epilogue, which is most of a small
+// launch.  (d 256, ffn 688: one split of O's four K blocks and two of down's eleven took 91 us a forward of 16 to 80 rows, four
+// of each 86, four and eight 87.)
 int auto_split_residual(int tiles, int k) {
+  const int kb = (k + 63) / 64;
   int s = 8;
-  while (s > 1 && tiles * s > kSms) s >>= 1;
-  return capped_split(s, k);
+  while (s > 1 && (tiles * s > kSms || s > kb || (s > 4 && 4 * s > kb))) s >>= 1;
+  return s;
 }
 // QKV: its finishing pass reads every split's partial sums.  One CTA per SM against two, eight layers: 36 tiles (4 splits, not 8)
 // 1018 -> 1007 us at 32 rows, 1328 -> 1282 at 128, 1591 -> 1555 at 192; 96 tiles (1, not 3) 968 -> 980, 1248 -> 1228, 1543 -> 1522.
