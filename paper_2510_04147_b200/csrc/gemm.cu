@@ -516,43 +516,23 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ 
           scratch[j * kEpiPitch + lrow] = live ? x : -INFINITY;
         }
         epi_bar_sync(group);
-        float m = -INFINITY, sum = 0.f;
-        int arg = 0x7fffffff;
         float x[32];
 #pragma unroll
         for (int q4 = 0; q4 < 8; ++q4) {
           const float4 t4 = *reinterpret_cast<const float4*>(scratch + rr * kEpiPitch + qf + q4 * 4);
           x[q4 * 4] = t4.x; x[q4 * 4 + 1] = t4.y; x[q4 * 4 + 2] = t4.z; x[q4 * 4 + 3] = t4.w;
         }
-#pragma unroll
-        for (int j = 0; j < 32; ++j)
-          if (x[j] > m) { m = x[j]; arg = tile * kTileM + qf + j; }
-        if (m != -INFINITY) {
-#pragma unroll
-          for (int j = 0; j < 32; ++j) sum += expf(x[j] - m);          // (exp(-inf) = 0 for dead entries)
-        }
+        LmStat st = lm_quarter(x, tile * kTileM + qf);
 #pragma unroll
         for (int o = 1; o <= 2; o <<= 1) {                               // quarters: (0 + 1), (2 + 3), then the pairs
-          const float om = __shfl_xor_sync(0xffffffffu, m, o);
-          const float os = __shfl_xor_sync(0xffffffffu, sum, o);
-          const int oa = __shfl_xor_sync(0xffffffffu, arg, o);
-          // the same value from both partners: the lower quarter's (maximum, index) wins a tie
-          const bool lower = (et & o) == 0;
-          const float m_lo = lower ? m : om, s_lo = lower ? sum : os, m_hi = lower ? om : m, s_hi = lower ? os : sum;
-          const int a_lo = lower ? arg : oa, a_hi = lower ? oa : arg;
-          const float M = fmaxf(m_lo, m_hi);
-          float S = 0.f;
-          if (m_lo != -INFINITY) S += s_lo * expf(m_lo - M);
-          if (m_hi != -INFINITY) S += s_hi * expf(m_hi - M);
-          arg = (m_hi > m_lo) ? a_hi : a_lo;
-          m = M;
-          sum = S;
+          const LmStat other{__shfl_xor_sync(0xffffffffu, st.m, o), __shfl_xor_sync(0xffffffffu, st.sum, o), __shfl_xor_sync(0xffffffffu, st.arg, o)};
+          st = (et & o) == 0 ? lm_merge(st, other) : lm_merge(other, st);
         }
         if ((et & 3) == 0 && c0 + rr < rows_here) {
           const size_t o = (size_t)tile * p.R + row0 + c0 + rr;
-          p.tile_max[o] = m;
-          p.tile_sum[o] = sum;
-          p.tile_arg[o] = arg;
+          p.tile_max[o] = st.m;
+          p.tile_sum[o] = st.sum;
+          p.tile_arg[o] = st.arg;
         }
         if (p.topk > 0) {
           // The quarter's largest entries, sorted (value descending, lower index first): an insertion only where an entry
@@ -563,18 +543,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ 
 #pragma unroll
           for (int r = 0; r < kLmTopKMax; ++r) { tv[r] = -INFINITY; ti[r] = 0x7fffffff; }
 #pragma unroll
-          for (int j = 0; j < 32; ++j) {
-            if (x[j] > tv[kLmTopKMax - 1]) {
-              const int idx = tile * kTileM + qf + j;
-#pragma unroll
-              for (int r = kLmTopKMax - 1; r > 0; --r) {                 // from the back: what is smaller moves down a place
-                const bool below = x[j] > tv[r - 1], here = !below && x[j] > tv[r];
-                if (below) { tv[r] = tv[r - 1]; ti[r] = ti[r - 1]; }
-                else if (here) { tv[r] = x[j]; ti[r] = idx; }
-              }
-              if (x[j] > tv[0]) { tv[0] = x[j]; ti[0] = idx; }
-            }
-          }
+          for (int j = 0; j < 32; ++j) lm_insert(tv, ti, x[j], tile * kTileM + qf + j);
           // the row's list from the four quarters' heads: one round per rank
           const bool put = c0 + rr < rows_here;
           const size_t o = ((size_t)tile * p.R + row0 + c0 + rr) * kLmTopKMax;

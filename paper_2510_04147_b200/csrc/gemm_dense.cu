@@ -11,8 +11,8 @@
 // loop of the next.  Tiles are walked rows first, so that the CTAs in flight share a few weight tiles and all of the
 // activations through L2.
 //
-// Epilogues: EPI_QKV (rotary embedding; q rows and k and v rows to their buffers and the K/V cache), EPI_SWIGLU and
-// EPI_RESIDUAL as in gemm.cu.  Two warpgroups share a tile's columns: group g of a 256-feature tile has the 128-feature
+// Epilogues: EPI_QKV (rotary embedding; q rows and k and v rows to their buffers and the K/V cache), EPI_SWIGLU, EPI_RESIDUAL and
+// EPI_LMHEAD as in gemm.cu.  Two warpgroups share a tile's columns: group g of a 256-feature tile has the 128-feature
 // half g, of a 128-feature tile the columns [32 g, +32) and 64 + [32 g, +32) - either way 32-column pieces together with
 // the piece 64 columns on, the rotary partner or the `up` of the `gate`.
 //
@@ -75,6 +75,14 @@ struct DenseParams {
   int sq_out_stride;
   // EPI_QKV
   QkvOut qkv;
+  // EPI_LMHEAD
+  float* tile_max;
+  float* tile_sum;
+  int* tile_arg;
+  int topk;
+  float* tile_topv;
+  int* tile_topi;
+  int mask_id;
 };
 
 __device__ __forceinline__ uint32_t smem_addr(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
@@ -385,6 +393,60 @@ gemm_dense_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant
         }
         inv = rsqrtf(ss / (float)p.norm_dim + p.norm_eps);
       }
+      if constexpr (kEpi == EPI_LMHEAD) {
+        // The group's half of the features is one vocabulary tile, all of a row's entries in one thread, a quarter at a time.
+        const int buf = nth % kBufs, v_tile = (n_base >> 7) + group, v0 = v_tile * 128;
+        if (ok) ok = mbar_wait(smem_addr(&acc_full[buf]), (uint32_t)((nth / kBufs) & 1), abort_flag, p.wait_limit_ns);
+        ok = __all_sync(0xffffffffu, ok);
+        ++nth;
+        if (!ok) continue;
+        tc_fence_after();
+        const uint32_t taddr = tmem_base + (uint32_t)(buf * kFeat + 128 * group) + ((uint32_t)(quad * 32) << 16);
+        const bool some_dead = v0 + 128 > p.N || (p.mask_id >= v0 && p.mask_id < v0 + 128);
+        LmStat st[4];
+        float tv[kLmTopKMax];
+        int ti[kLmTopKMax];
+#pragma unroll
+        for (int r = 0; r < kLmTopKMax; ++r) { tv[r] = -INFINITY; ti[r] = 0x7fffffff; }
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+          uint32_t r1[16], r2[16];
+          tmem_ld16_issue(taddr + 32 * q, r1);
+          tmem_ld16_issue(taddr + 32 * q + 16, r2);
+          tmem_ld_wait(r1);
+          tmem_ld_wait(r2);
+          float x[32];
+#pragma unroll
+          for (int j = 0; j < 16; ++j) {
+            x[j] = p.sq != nullptr ? __uint_as_float(r1[j]) * inv : __uint_as_float(r1[j]);
+            x[16 + j] = p.sq != nullptr ? __uint_as_float(r2[j]) * inv : __uint_as_float(r2[j]);
+          }
+          if (some_dead) {
+#pragma unroll
+            for (int j = 0; j < 32; ++j)
+              if (v0 + 32 * q + j >= p.N || v0 + 32 * q + j == p.mask_id) x[j] = -INFINITY;
+          }
+          st[q] = lm_quarter(x, v0 + 32 * q);
+          if (p.topk > 0) {
+#pragma unroll
+            for (int j = 0; j < 32; ++j) lm_insert(tv, ti, x[j], v0 + 32 * q + j);
+          }
+        }
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) mbar_arrive_leader(smem_addr(&acc_empty[buf]));
+        if (live && v0 < p.N) {
+          const LmStat s = lm_merge(lm_merge(st[0], st[1]), lm_merge(st[2], st[3]));
+          const size_t o = (size_t)v_tile * p.R + row;
+          p.tile_max[o] = s.m;
+          p.tile_sum[o] = s.sum;
+          p.tile_arg[o] = s.arg;
+#pragma unroll
+          for (int r = 0; r < kLmTopKMax; ++r)
+            if (r < p.topk) { p.tile_topv[o * kLmTopKMax + r] = tv[r]; p.tile_topi[o * kLmTopKMax + r] = ti[r]; }
+        }
+        continue;
+      }
       float run[kCh][2][32];                 // running sums over the K ranges; EPI_RESIDUAL: on top of the residual stream
       if (kEpi == EPI_RESIDUAL) {
         float4 t[2 * kCh][8];                // all pieces in flight together
@@ -605,6 +667,8 @@ int launch_gemm_dense(cudaStream_t st, const GemmArgs& g) {
     if ((g.N & 3) || !g.h || !g.hb || !g.gain || !g.sq_out) return -2;
   } else if (g.epi == EPI_SWIGLU) {
     if ((g.N % 128) || g.splits != 1) return -2;
+  } else if (g.epi == EPI_LMHEAD) {
+    if (g.splits != 1 || !g.tile_max || !g.tile_sum || !g.tile_arg || g.topk < 0 || g.topk > kLmTopKMax || (g.topk > 0 && (!g.tile_topv || !g.tile_topi))) return -2;
   } else if (g.epi == EPI_QKV) {
     if (!g.qkv || (g.qkv->hd != 64 && g.qkv->hd != 128) || !g.sq) return -2;
   } else {
@@ -619,6 +683,8 @@ int launch_gemm_dense(cudaStream_t st, const GemmArgs& g) {
   p.act = g.act; p.act_pitch = g.act_pitch;
   p.h = g.h; p.hb = g.hb; p.gain = g.gain; p.sq_out = g.sq_out; p.sq_out_stride = g.sq_out_stride;
   if (g.qkv) p.qkv = *g.qkv;
+  p.tile_max = g.tile_max; p.tile_sum = g.tile_sum; p.tile_arg = g.tile_arg; p.topk = g.topk; p.tile_topv = g.tile_topv; p.tile_topi = g.tile_topi;
+  p.mask_id = g.mask_id;
   static int sm_count[kMaxDevices] = {};
   const int dev = device_slot();
   if (dev < 0) return -4;
@@ -638,6 +704,7 @@ int launch_gemm_dense(cudaStream_t st, const GemmArgs& g) {
   const bool narrow = g.epi == EPI_RESIDUAL ? waves128 * (60 + 3 * kb) < waves256 * (240 + 4 * kb)
                                             : !(g.epi == EPI_QKV && g.qkv->hd == 64) && waves128 * 6 < waves256 * 10;
   switch (g.epi) {
+    case EPI_LMHEAD: return launch<256, EPI_LMHEAD>(st, g, p, sms, dev);
     case EPI_QKV: return narrow ? launch<128, EPI_QKV>(st, g, p, sms, dev) : launch<256, EPI_QKV>(st, g, p, sms, dev);
     case EPI_SWIGLU: return narrow ? launch<128, EPI_SWIGLU>(st, g, p, sms, dev) : launch<256, EPI_SWIGLU>(st, g, p, sms, dev);
     default: return narrow ? launch<128, EPI_RESIDUAL>(st, g, p, sms, dev) : launch<256, EPI_RESIDUAL>(st, g, p, sms, dev);

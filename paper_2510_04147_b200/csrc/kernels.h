@@ -315,6 +315,42 @@ int encode_tmap_bf16_3d(void* map_out, const void* base, uint64_t cols, uint64_t
                         uint64_t plane_pitch, uint32_t box_rows);
 int encode_tmap_bf16_2d(void* map_out, const void* base, uint64_t rows, uint64_t cols, uint64_t pitch_elems, uint32_t box_rows);
 
+#ifdef __CUDACC__
+// ---- what the LM head keeps of a vocabulary tile of 128 entries, per row: maximum with the lowest index among equals, sum of
+// exp(x - its maximum) and, where asked, the largest entries.  A tile is worked on in quarters of 32 entries, merged (0 + 1) + (2 + 3),
+// in every kernel and whoever has the quarters: the value depends on the tile alone.
+struct LmStat { float m, sum; int arg; };
+__device__ __forceinline__ LmStat lm_quarter(const float (&x)[32], int first) {
+  LmStat s{-INFINITY, 0.f, 0x7fffffff};
+#pragma unroll
+  for (int j = 0; j < 32; ++j)
+    if (x[j] > s.m) { s.m = x[j]; s.arg = first + j; }
+  if (s.m != -INFINITY) {
+#pragma unroll
+    for (int j = 0; j < 32; ++j) s.sum = __fadd_rn(s.sum, expf(x[j] - s.m));              // (exp(-inf) = 0 for dead entries)
+  }
+  return s;
+}
+// the same value from both partners: the lower quarter's (maximum, index) wins a tie
+__device__ __forceinline__ LmStat lm_merge(const LmStat& lo, const LmStat& hi) {
+  LmStat s{fmaxf(lo.m, hi.m), 0.f, hi.m > lo.m ? hi.arg : lo.arg};
+  if (lo.m != -INFINITY) s.sum = __fmaf_rn(lo.sum, expf(lo.m - s.m), s.sum);
+  if (hi.m != -INFINITY) s.sum = __fmaf_rn(hi.sum, expf(hi.m - s.m), s.sum);
+  return s;
+}
+// sorted lists (value descending, lower index first): an insertion only where an entry beats the last of the list
+__device__ __forceinline__ void lm_insert(float (&tv)[kLmTopKMax], int (&ti)[kLmTopKMax], float x, int idx) {
+  if (!(x > tv[kLmTopKMax - 1])) return;
+#pragma unroll
+  for (int r = kLmTopKMax - 1; r > 0; --r) {                 // from the back: what is smaller moves down a place
+    const bool below = x > tv[r - 1], here = !below && x > tv[r];
+    if (below) { tv[r] = tv[r - 1]; ti[r] = ti[r - 1]; }
+    else if (here) { tv[r] = x; ti[r] = idx; }
+  }
+  if (x > tv[0]) { tv[0] = x; ti[0] = idx; }
+}
+#endif
+
 // ---------------------------------------------------------------- tree build / acceptance
 // Words of BlockState::mirror per sequence, written by the acceptance kernel
 enum { MIRROR_REMAINING = 0, MIRROR_REMAINING_NXT, MIRROR_HAS_DRAFTS, MIRROR_LAST_ACCEPT, MIRROR_N_CAND, kMirrorWords };

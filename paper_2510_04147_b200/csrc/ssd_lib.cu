@@ -362,8 +362,8 @@ int run_gemm(ssd_ctx* c, GemmArgs g, int fam, int sub = -1) {
   return SSD_OK;
 }
 
-int run_gemm_dense(ssd_ctx* c, GemmArgs g, int sub) {
-  Scope sc(c, SSD_PROF_GEMM, (double)g.N * g.K * 2.0, 1, sub);
+int run_gemm_dense(ssd_ctx* c, GemmArgs g, int sub, int fam = SSD_PROF_GEMM) {
+  Scope sc(c, fam, (double)g.N * g.K * 2.0, 1, sub);
   g.err_flag = c->flags;
   g.wait_limit_ns = (unsigned long long)c->wait_limit_us * 1000ull;
   const int rc = launch_gemm_dense(c->st, g);
@@ -590,7 +590,11 @@ int forward(ssd_ctx* c, int kind, const int* ids_dev, int R, RowMap map, int n_s
     } else {
       g.epi = EPI_LMHEAD; g.tile_max = c->tile_max; g.tile_sum = c->tile_sum; g.tile_arg = c->tile_arg;
       if (range.topk > 0) { g.topk = range.topk; g.tile_topv = c->tile_topv; g.tile_topi = c->tile_topi; }
-      int rc = run_gemm(c, g, SSD_PROF_LMHEAD);
+      // The dense kernel has the statistics of a tile under the next one's main loop; where its 256-row tiles are filled.  us,
+      // skinny / dense, V 126464, d 4096: 32 rows 164 / 192, 128 rows 202 / 202, 160 223 / 211, 192 246 / 220, 256 287 / 228, 320
+      // 350 / 385, 512 497 / 402; V 152064, d 3584: 128 rows 221 / 233, 256 288 / 252, 320 395 / 418.
+      const bool dense_lm = 3 * R > 2 * c->dense_rows && (R <= 256 || R * 16 >= (R + 255) / 256 * 256 * 13);
+      int rc = dense_lm ? run_gemm_dense(c, g, -1, SSD_PROF_LMHEAD) : run_gemm(c, g, SSD_PROF_LMHEAD);
       if (rc) return rc;
       Scope sc(c, SSD_PROF_LMHEAD, (double)gemm_tiles(c->V) * R * 12.0, range.topk > 0 ? 2 : 1);
       launch_lm_merge(c->st, c->tile_max, c->tile_sum, c->tile_arg, gemm_tiles(c->V), R, c->V, row_wanted, c->tok, c->conf);
