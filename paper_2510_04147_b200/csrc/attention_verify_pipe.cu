@@ -32,7 +32,10 @@
 // 3400 clocks (clock64 at each step, 4096 keys) the scores' maximum took 580, the wait for O += P V 425, exponentials, sums and P
 // 1850, of which the special-function unit accounts for 1024.  Taken out: the visibility test of every key (masked scores become
 // -inf where they are loaded) and that wait: 4 sequences of 4096 keys 77 -> 72 us at 128 rows each, 1536 keys 24.2 -> 22.9.
-// Keeping all 64 scores of a thread in registers, four threads to a row, or even and odd tiles in two streams were no faster.
+// Four threads to a row, or even and odd tiles in two streams, were no faster.  A thread keeps its scores in registers from the maximum
+// to the exponentials, 64 of them under 128 rows, where the outputs of parts in one CTA do not need those registers (kShared; with
+// them spilled, 28 heads at 320 rows 35 -> 49 us): read twice / kept, us a layer: 4 sequences of 4096 keys, 128 rows each 88 / 79; 8 of 509 keys, 96
+// rows each 50.5 / 42.1; one sequence, 512 keys, 128 rows 17.3 / 14.7; 1024 keys, 28 heads, 128 rows 17.9 / 15.6.
 // us per layer in the live stream (the forms before it, which summed and rotated the projection's split-K partials themselves, in
 // brackets; finishing q, k and v is now a pass of 3 to 10 us): one sequence, 512 keys, 32 / 64 / 128 rows 10 (15) / 13 (20) /
 // 19 (32); 1536 keys, 128 rows 23 (43); 8 sequences of 512 keys 27 (38); 4 of 4096 keys, 64 / 128 rows each 56 (83) / 72
@@ -41,6 +44,8 @@
 
 #include <cuda.h>
 #include <string.h>
+
+#include <atomic>
 
 namespace ssd {
 
@@ -238,9 +243,12 @@ __device__ __forceinline__ Merge merge_of(float m_before, float m_next) {
   g.next = ex2(m_next - use);
   return g;
 }
+template <int N>
+struct IntC { static constexpr int value = N; };
 __device__ __forceinline__ float merged(const Merge& g, float before, float next) { return __fmaf_rn(next, g.next, __fmul_rn(before, g.before)); }
 
-template <int QT>
+// kShared: a CTA has several parts (n_ctas < n_parts)
+template <int QT, bool kShared>
 __global__ void __launch_bounds__(kPipeBlock, 1)
 attn_verify_pipe_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_constant__ CUtensorMap tmLK,
                         const __grid_constant__ CUtensorMap tmLV, const __grid_constant__ CUtensorMap tmK,
@@ -439,9 +447,9 @@ attn_verify_pipe_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
     // over through mbarriers, so that no thread waits for the MMA issue.
     constexpr int KPT = QT / 2;                           // keys of a tile per thread
     constexpr int NCH = KPT / 16;                         // 16-key chunks per thread
-    // A thread takes its keys in passes of at most 32 (its scores then fit in registers): one pass for tiles of 32
-    // or 64 rows, whose scores stay in registers from the maximum to the exponentials; two for 128 rows, read again.
-    constexpr int HK = KPT < 32 ? KPT : 32, NP = KPT / HK, NCP = HK / 16;
+    // A thread takes its keys in one pass, its scores in registers from the maximum to the exponentials; in two, whose scores are
+    // read again, where 128 rows meet parts that share the CTA.  (The output is rescaled 32 columns at a time.)
+    constexpr int HK = kShared && KPT > 32 ? 32 : KPT, NP = KPT / HK, NCP = HK / 16, RK = KPT < 32 ? KPT : 32;
     const int lt = tid & 127, hw = tid >> 7;
     const int cw = lt / QT, row = lt % QT;
     const uint32_t lane_addr = (uint32_t)((warp & 3) * 32) << 16;   // warps w and w + 4 read TMEM lanes 32 (w & 3) ...
@@ -457,7 +465,7 @@ attn_verify_pipe_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
     float acc[KPT], acc_m = -INFINITY, acc_l = 0.f;
     bool have = false;
     auto part_done = [&](float m, float l) {              // the part whose output stands in tensor memory
-      const bool fold = have;
+      const bool fold = kShared && have;
       const Merge g2 = merge_of(acc_m, m);
 #pragma unroll
       for (int ch = 0; ch < NCH; ++ch) {
@@ -525,10 +533,8 @@ attn_verify_pipe_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
       sMaxU[(hw * 4 + cw) * 128 + row] = m_loc;
       ok = softmax_barrier_and(ok);                         // the one meeting of a tile; also one decision for all
       if (!ok) { broke = true; break; }
-      if (u > 0) {                                          // (every chunk sum of the previous tile is visible now)
-        l_row = l_row * corr_prev + tile_sum(u - 1);
-      }
-      if (u == fresh_at && u < n_tiles) {                   // this tile starts a part: put the one before away
+      if (kShared && u > 0) l_row = l_row * corr_prev + tile_sum(u - 1);      // (every chunk sum of the previous tile is visible now)
+      if (kShared && u == fresh_at) {                   // this tile starts a part: put the one before away
         fresh_at = g.begin(++next_part) - first;
         ok = mbar_wait(bar_o0 + 8u * (uint32_t)((u - 1) & 1), (uint32_t)(((u - 1) >> 1) & 1), abort_flag);
         tc_fence_after();
@@ -556,19 +562,19 @@ attn_verify_pipe_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
       }
       if (ok && rescale) {
 #pragma unroll
-        for (int pass = 0; pass < NP; ++pass) {
-          uint32_t ov[HK];
+        for (int pass = 0; pass < KPT / RK; ++pass) {
+          uint32_t ov[RK];
 #pragma unroll
-          for (int ch = 0; ch < NCP; ++ch) tmem_ld16_issue(tmem_O + lane_addr + col0 + pass * HK + ch * 16, &ov[ch * 16]);
+          for (int ch = 0; ch < RK / 16; ++ch) tmem_ld16_issue(tmem_O + lane_addr + col0 + pass * RK + ch * 16, &ov[ch * 16]);
           tmem_ld_wait();
 #pragma unroll
-          for (int ch = 0; ch < NCP; ++ch) keep16(&ov[ch * 16]);
+          for (int ch = 0; ch < RK / 16; ++ch) keep16(&ov[ch * 16]);
 #pragma unroll
-          for (int ch = 0; ch < NCP; ++ch) {
+          for (int ch = 0; ch < RK / 16; ++ch) {
             float v[16];
 #pragma unroll
             for (int j = 0; j < 16; ++j) v[j] = __uint_as_float(ov[ch * 16 + j]) * corr;
-            tmem_st16(tmem_O + lane_addr + col0 + pass * HK + ch * 16, v);
+            tmem_st16(tmem_O + lane_addr + col0 + pass * RK + ch * 16, v);
           }
         }
       }
@@ -592,7 +598,7 @@ attn_verify_pipe_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
           sSumU[(c0 >> 4) * 128 + row] = csum[ch];          // chunk index = c0 / 16
           uint32_t packed[8];
 #pragma unroll
-          for (int j = 0; j < 8; ++j) packed[j] = row_live ? pack_bf16(p[ch * 16 + 2 * j], p[ch * 16 + 2 * j + 1]) : 0u;
+          for (int j = 0; j < 8; ++j) packed[j] = pack_bf16(p[ch * 16 + 2 * j], p[ch * 16 + 2 * j + 1]);
           if (kTmemP) {
             if (ok) tmem_st8(tmem_P + (uint32_t)(u & 1) * 64u + lane_addr + (uint32_t)(c0 >> 1), packed);
           } else {                                          // P, in every copy of the row
@@ -612,6 +618,7 @@ attn_verify_pipe_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
       tc_fence_before();
       __syncwarp();
       if (lane == 0) mbar_arrive(bar_p);
+      if (!kShared && u > 0) l_row = l_row * corr_prev + tile_sum(u - 1);     // (not before the exponentials: nothing waits for it)
       corr_prev = corr;
       m_row = m_new;
     }
@@ -623,7 +630,7 @@ attn_verify_pipe_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
     }
     ok = __all_sync(0xffffffffu, ok ? 1 : 0) != 0;
     // this CTA's last part; a CTA that has not the first part of all hands two parts on as two entries
-    const bool two = have && rank > 0;
+    const bool two = kShared && have && rank > 0;
     if (ok && !two) part_done(m_row, l_row);
     if (ok && g.n_ctas == 1) {
       // every copy of a row holds the same O row: a thread normalises and stores the columns it owns, [col0, +KPT)
@@ -712,10 +719,18 @@ attn_verify_pipe_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
   }
 }
 
-template <int QT>
+template <int QT, bool kShared>
 cudaError_t launch_pipe(cudaStream_t st, dim3 grid, size_t smem, const CUtensorMap (&tm)[5], const AttnArgs& a, const PipeShape& g,
                         float scale_log2) {
-  return launch_pdl_cluster(attn_verify_pipe_kernel<QT>, grid, dim3(kPipeBlock), smem, st, (unsigned)g.n_ctas, tm[0], tm[1], tm[2], tm[3], tm[4], a, g,
+  static std::atomic<bool> attr_set[kMaxDevices] = {};        // the shared-memory opt-in is per device
+  const int dev = device_slot();
+  if (dev < 0) return cudaErrorInvalidDevice;
+  if (!attr_set[dev]) {
+    const cudaError_t e = cudaFuncSetAttribute(attn_verify_pipe_kernel<QT, kShared>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+    attr_set[dev] = true;
+  }
+  return launch_pdl_cluster(attn_verify_pipe_kernel<QT, kShared>, grid, dim3(kPipeBlock), smem, st, (unsigned)g.n_ctas, tm[0], tm[1], tm[2], tm[3], tm[4], a, g,
                             scale_log2);
 }
 
@@ -752,16 +767,6 @@ int launch_attention_verify_pipe(cudaStream_t st, const AttnArgs& a, int n_parts
   }
   const float scale_log2 = (1.0f / sqrtf((float)a.hd)) * 1.4426950408889634f;
   const size_t smem = (size_t)kTileBytes * (2 + kStagesK + kStagesV) + 16384 + 128 + 1024;   // Q, P, K and V stages, softmax exchange
-  static bool attr_set[kMaxDevices] = {};        // the shared-memory opt-in is per device
-  const int dev = device_slot();
-  if (dev < 0) return -4;
-  if (!attr_set[dev]) {
-    if (cudaFuncSetAttribute(attn_verify_pipe_kernel<32>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess ||
-        cudaFuncSetAttribute(attn_verify_pipe_kernel<64>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess ||
-        cudaFuncSetAttribute(attn_verify_pipe_kernel<128>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
-      return -4;
-    attr_set[dev] = true;
-  }
   alignas(64) CUtensorMap tm[5];
   const uint64_t planes = (uint64_t)a.cache_rows * kHD / a.kv_head_stride;       // (sequence, kv head) pairs
   const uint64_t bound = (uint64_t)(a.S + a.hole_len > 0 ? a.S + a.hole_len : 1);
@@ -773,10 +778,11 @@ int launch_attention_verify_pipe(cudaStream_t st, const AttnArgs& a, int n_parts
       encode_tmap_bf16_3d(&tm[4], a.cache_v, kHD, bound, planes, kHD, a.kv_head_stride, kKeys) != 0)
     return -4;
   const dim3 grid(a.H * g.n_ctas, a.n_seq_slots * q_tiles);
-  cudaError_t e;
-  if (qt_rows == 32) e = launch_pipe<32>(st, grid, smem, tm, a, g, scale_log2);
-  else if (qt_rows == 64) e = launch_pipe<64>(st, grid, smem, tm, a, g, scale_log2);
-  else e = launch_pipe<128>(st, grid, smem, tm, a, g, scale_log2);
+  const auto launch = [&](auto qt) {
+    constexpr int QT = decltype(qt)::value;
+    return g.n_ctas < g.n_parts ? launch_pipe<QT, true>(st, grid, smem, tm, a, g, scale_log2) : launch_pipe<QT, false>(st, grid, smem, tm, a, g, scale_log2);
+  };
+  const cudaError_t e = qt_rows == 32 ? launch(IntC<32>()) : qt_rows == 64 ? launch(IntC<64>()) : launch(IntC<128>());
   return e == cudaSuccess ? 0 : -4;
 }
 
