@@ -313,15 +313,16 @@ int ssd_profile_read(ssd_ctx* ctx, int64_t* launches, double* milliseconds, doub
  *        dimension 128, nodes of up to 128 rows), the default; 0 = always the mma.sync form;
  *   "attn_pipe_ctas", "attn_pipe_keys" with attn_impl 1: a prefilled batch that gives at least attn_pipe_ctas
  *        (default 64, from 1024 cached keys on 75) pairs (head, sequence) - batch * heads - has one CTA per pair walk all key
- *        tiles, instead of cutting them into parts that a cluster can share; one sequence is faster with its key parts side by side.  attn_pipe_keys (default 1; 0 = never) is the shortest prefix that may take it.
+ *        tiles, instead of cutting them into parts that a cluster can share; one sequence is faster with its key parts side by
+ *        side.  attn_pipe_keys (default 1; 0 = never) is the shortest prefix that may take it.
  *        The two forms sum in different orders, so a sequence's bits depend on the prefilled batch SIZE - never
  *        on the other sequences' contents, on the node count, or on which sequences are still unfinished;
  *   "dense_rows" in forwards of more rows than this (default 240) a projection may run as a dense contraction instead
  *        of a stream of the weights, and from two thirds of it on the LM head likewise and (up to 256 rows) a projection with its
  *        features shared out evenly over the SMs, where its size makes that the faster one; the results are bit-identical
  *        either way;
- *   "two_sm_rows" the QKV, gate/up and LM-head projections run pairs of weight tiles as ONE tcgen05.mma
- *        with cta_group::2 (two CTAs of a cluster, M = 256, each SM holding half of the activation tile)
+ *   "two_sm_rows" the QKV, gate/up and LM-head projections, and O and down where their clusters find room, run pairs of weight
+ *        tiles as ONE tcgen05.mma with cta_group::2 (two CTAs, M = 256, each SM holding half of the activation tile)
  *        from this many padded rows per launch on; 0 = never; default 128, where it starts to pay.  The results
  *        are bit-identical either way;
  *   "fuse_commit" 1 = a block's commit is folded into the next block's first forward (default); 0 = a
