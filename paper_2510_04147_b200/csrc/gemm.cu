@@ -398,21 +398,14 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ 
     pdl_wait();                                // outputs may still be read by the predecessor
     const int et = (threadIdx.x - 64) & 127;   // 0..127 among the group's threads
     if (p.sq != nullptr) {
-      // fused RMSNorm, consumer side: 1/rms of every row from the producers' sums of squares
+      // fused RMSNorm, consumer side: 1/rms of every row from the producers' per-tile sums of squares
       // (summed in slot order), computed while the main loop still runs
       for (int rr = threadIdx.x - 64; rr < p.npad; rr += kEpiThreads) {
         float inv = 0.f;
         if (row0 + rr < p.R) {
           const float* q = p.sq + (size_t)(row0 + rr) * p.sq_stride;
           float ss = 0.f;
-          if (((p.sq_count | p.sq_stride) & 3) == 0) {
-            for (int t = 0; t < p.sq_count; t += 4) {
-              const float4 v = *reinterpret_cast<const float4*>(q + t);
-              ss += v.x; ss += v.y; ss += v.z; ss += v.w;
-            }
-          } else {
-            for (int t = 0; t < p.sq_count; ++t) ss += q[t];
-          }
+          for (int t = 0; t < p.sq_count; ++t) ss += q[t];
           inv = rsqrtf(ss / (float)p.norm_dim + p.norm_eps);
         }
         s_inv[rr] = inv;
@@ -585,7 +578,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ 
     // features] in shared memory;
     // after a cluster barrier CTA `rank` owns the rows rank, rank + splits, ... (a row per warp, a
     // lane per four features): it adds the partials in split order to the residual stream, writes h,
-    // bf16(h * gain) and the row's sums of squares, one for each 64 features.  A second barrier frees the staging
+    // bf16(h * gain) and the tile's sum of squares of the row.  A second barrier frees the staging
     // buffer.  Every thread of every CTA passes both barriers of every pass, also after an error.
     const bool epi_warp = warp >= 2;
     const int quad = warp & 3, group = (warp - 2) >> 2;
@@ -604,7 +597,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ 
     int pass_rows = (p.stages * (kWTileBytes + x_tile_bytes)) / (kEpiPitch * 4) / 32 * 32;
     const int npad32 = (p.npad + 31) & ~31;               // whole chunks (TMEM holds a power of two >= 32 columns)
     if (pass_rows > npad32) pass_rows = npad32;
-    // h, bf16(h * gain) and the row's sums of squares, one for each 64 features (EPI_SUM: the sums)
+    // h, bf16(h * gain) and the tile's sum of squares of the row (EPI_SUM: the sums)
     auto store = [&](int row, const float4& acc) {
       if (!resid) {
         float* dst = p.out + (size_t)(row0 + row) * p.N + n_base + f4;
@@ -628,9 +621,8 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ 
         ss = sumsq4(acc);
       }
 #pragma unroll
-      for (int o = 8; o > 0; o >>= 1) ss += __shfl_xor_sync(0xffffffffu, ss, o);       // one sum for each 64 features
-      const int slot = (n_base + f4) >> 6;
-      if ((lane & 15) == 0 && slot * 64 < p.N) p.sq_out[(size_t)(row0 + row) * p.sq_out_stride + slot] = ss;
+      for (int o = 16; o > 0; o >>= 1) ss += __shfl_xor_sync(0xffffffffu, ss, o);
+      if (lane == 0) p.sq_out[(size_t)(row0 + row) * p.sq_out_stride + tile] = ss;
     };
     // The rows of this CTA (rank, rank + n_ranks, ...) go round the warps; a warp takes kU of them at a time with all
     // kU * kQ remote reads in flight (kQ >= n_ranks) and adds each row's partials in split order.

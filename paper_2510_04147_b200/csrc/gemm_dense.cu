@@ -45,12 +45,11 @@ constexpr int kTransBytes = kEpiThreads / 32 * kTransWarp;
 template <int kFeat>
 struct Cfg {
   static constexpr int kStageBytes = kXBytes + kFeat / 2 * kBlockK * 2;
-  static constexpr int kStages = kFeat == 128 ? 7 : 6;
+  static constexpr int kStages = kFeat == 256 ? 6 : 7;
   static constexpr int kBufs = 512 / kFeat;            // accumulators
-  static constexpr int kCh = (kFeat + 127) / 128;      // pairs of 32-column pieces per epilogue thread
-  static constexpr int kSlots = kFeat / 64;            // 64-feature slots of the sums of squares
-  static constexpr int kSumPitch = 8 * kSlots + 1;     // floats per row of their exchange between the groups
-  static constexpr int kSumBytes = kFeat < 256 ? 2 * 128 * kSumPitch * 4 : 0;
+  static constexpr int kCh = kFeat / 128;              // 32-column pieces (with their partners) per epilogue thread
+  static constexpr int kSumPitch = 9;                  // floats per row of the sum-of-squares exchange (8 + padding)
+  static constexpr int kSumBytes = kCh == 1 ? 2 * 128 * kSumPitch * 4 : 0;
   static constexpr int kSmem = kStages * kStageBytes + kTransBytes + kSumBytes + 256 /*barriers*/ + 1024 /*alignment slack*/;
   static_assert(kSmem <= 227 * 1024, "shared memory");
 };
@@ -225,7 +224,7 @@ gemm_dense_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant
   extern __shared__ uint8_t smem_dyn[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_dyn) + 1023) & ~(uintptr_t)1023);
   uint8_t* sTrans = smem + kStages * kStageBytes;
-  float* sSum = reinterpret_cast<float*>(sTrans + kTransBytes);        // EPI_RESIDUAL: [2 tiles][128 rows][kSumPitch]
+  float* sSum = reinterpret_cast<float*>(sTrans + kTransBytes);        // [2 tiles][128 rows][kSumPitch]
   uint64_t* bars = reinterpret_cast<uint64_t*>(sTrans + kTransBytes + kSumBytes);
   uint64_t* full_bar = bars;                       // leader: both CTAs' bytes of a stage
   uint64_t* empty_bar = bars + kStages;            // each CTA: its stage may be refilled
@@ -280,29 +279,18 @@ gemm_dense_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant
       auto enter = [&](At& at) {             // first K block of a tile
         const int nt = at.tile / p.m_tiles, mt = at.tile - nt * p.m_tiles;
         // tile-contiguous weights: 128 rows per (128-feature tile, K block); a 128-feature tile is shared by the pair
-        // (192: three boxes of 32 rows, which lie in one weight tile each)
-        at.w_row = kFeat == 256 ? (nt * 2 + (int)crank) * n_kb * 128 : kFeat == 128 ? nt * n_kb * 128 + (int)crank * 64 : nt * 192 + (int)crank * 96;
+        at.w_row = kFeat == 256 ? (nt * 2 + (int)crank) * n_kb * 128 : nt * n_kb * 128 + (int)crank * 64;
         at.x_row = mt * kTileRows + (int)crank * 128;
       };
       auto next = [&](At& at) {
-        if (kFeat != 192) at.w_row += 128;
+        at.w_row += 128;
         if (++at.kb == n_kb) {
           at.kb = 0;
           at.tile += n_pairs;
           if (at.tile < total) enter(at);
         }
       };
-      auto load_w = [&](const At& at, int s) {
-        if constexpr (kFeat == 192) {
-#pragma unroll
-          for (int i = 0; i < 3; ++i) {
-            const int f = at.w_row + 32 * i;
-            tma_load_2d_pair(smem0 + s * kStageBytes + kXBytes + i * 32 * kBlockK * 2, &tmW, full0 + 8 * s, 0, ((f >> 7) * n_kb + at.kb) * 128 + (f & 127));
-          }
-        } else {
-          tma_load_2d_pair(smem0 + s * kStageBytes + kXBytes, &tmW, full0 + 8 * s, 0, at.w_row);
-        }
-      };
+      auto load_w = [&](const At& at, int s) { tma_load_2d_pair(smem0 + s * kStageBytes + kXBytes, &tmW, full0 + 8 * s, 0, at.w_row); };
       auto load_x = [&](const At& at, int s) { tma_load_2d_pair(smem0 + s * kStageBytes, &tmX, full0 + 8 * s, at.kb * kBlockK, at.x_row); };
       auto expect = [&](int s) { if (leader) mbar_expect_tx(full0 + 8 * s, 2u * kStageBytes); };
       // the weights depend on no earlier kernel: fill the ring with them before the dependency wait
@@ -390,13 +378,9 @@ gemm_dense_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant
       const int lr4 = lane >> 3, lc4 = 4 * (lane & 7);       // transposed form: row 4 i + lr4, columns from lc4
       // this thread's columns: piece c is [col(c), +32) together with [col(c) + 64, +32)
       auto col = [&](int c) -> int { return kFeat == 256 ? 128 * group + 32 * c : 32 * group; };
-      // EPI_RESIDUAL: 32-column pieces, half of a 64-feature slot each (256 features: both halves are in the thread, else the groups
-      // have one each)
-      constexpr int kPieces = kFeat == 256 ? 4 : kFeat / 64;
-      auto piece = [&](int e) -> int { return kFeat == 256 ? 128 * group + 32 * (e >> 1) + 64 * (e & 1) : 64 * e + 32 * group; };
       const bool live = row < p.R;
       float inv = 1.f;
-      if (p.sq != nullptr && live) {         // RMSNorm, consumer side: the producers' sums in slot order
+      if (p.sq != nullptr && live) {         // RMSNorm, consumer side: the producers' per-tile sums in slot order
         const float* q = p.sq + (size_t)row * p.sq_stride;
         float ss = 0.f;
         if (((p.sq_count | p.sq_stride) & 3) == 0) {
@@ -465,16 +449,16 @@ gemm_dense_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant
       }
       float run[kCh][2][32];                 // running sums over the K ranges; EPI_RESIDUAL: on top of the residual stream
       if (kEpi == EPI_RESIDUAL) {
-        float4 t[kPieces][8];                // all pieces in flight together
+        float4 t[2 * kCh][8];                // all pieces in flight together
 #pragma unroll
-        for (int e = 0; e < kPieces; ++e)
+        for (int e = 0; e < 2 * kCh; ++e)
 #pragma unroll
           for (int i = 0; i < 8; ++i) {
-            const int n = n_base + piece(e) + lc4, r = row0 + 4 * i + lr4;
+            const int n = n_base + col(e >> 1) + 64 * (e & 1) + lc4, r = row0 + 4 * i + lr4;
             t[e][i] = (r < p.R && n < p.N) ? *reinterpret_cast<const float4*>(p.h + (size_t)r * p.N + n) : make_float4(0.f, 0.f, 0.f, 0.f);
           }
 #pragma unroll
-        for (int e = 0; e < kPieces; ++e) lines_to_rows(trans, lane, t[e], run[e >> 1][e & 1]);
+        for (int e = 0; e < 2 * kCh; ++e) lines_to_rows(trans, lane, t[e], run[e >> 1][e & 1]);
       } else {
 #pragma unroll
         for (int c = 0; c < kCh; ++c)
@@ -488,36 +472,26 @@ gemm_dense_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant
         if (!ok) continue;
         tc_fence_after();
         const uint32_t taddr = tmem_base + (uint32_t)(buf * kFeat) + ((uint32_t)(quad * 32) << 16);
-        if constexpr (kEpi == EPI_RESIDUAL) {
 #pragma unroll
-          for (int e = 0; e < kPieces; ++e) {
-            uint32_t r1[16], r2[16];
-            tmem_ld16_issue(taddr + piece(e), r1);
-            tmem_ld16_issue(taddr + piece(e) + 16, r2);
-            tmem_ld_wait(r1);
-            tmem_ld_wait(r2);
+        for (int e = 0; e < 2 * kCh; ++e) {          // 16 columns and their partners at a time
+          const int c = e >> 1, j0 = (e & 1) * 16;
+          uint32_t r1[16], r2[16];
+          tmem_ld16_issue(taddr + col(c) + j0, r1);
+          tmem_ld16_issue(taddr + col(c) + j0 + 64, r2);
+          tmem_ld_wait(r1);
+          tmem_ld_wait(r2);
+          if (kEpi == EPI_RESIDUAL) {
 #pragma unroll
-            for (int j = 0; j < 16; ++j) { run[e >> 1][e & 1][j] += __uint_as_float(r1[j]); run[e >> 1][e & 1][16 + j] += __uint_as_float(r2[j]); }
-          }
-        } else {
+            for (int j = 0; j < 16; ++j) { run[c][0][j0 + j] += __uint_as_float(r1[j]); run[c][1][j0 + j] += __uint_as_float(r2[j]); }
+          } else if (kEpi == EPI_QKV) {
 #pragma unroll
-          for (int e = 0; e < 2 * kCh; ++e) {        // 16 columns and their partners at a time
-            const int c = e >> 1, j0 = (e & 1) * 16;
-            uint32_t r1[16], r2[16];
-            tmem_ld16_issue(taddr + col(c) + j0, r1);
-            tmem_ld16_issue(taddr + col(c) + j0 + 64, r2);
-            tmem_ld_wait(r1);
-            tmem_ld_wait(r2);
-            if (kEpi == EPI_QKV) {
-#pragma unroll
-              for (int j = 0; j < 16; ++j) {
-                run[c][0][j0 + j] = __fadd_rn(run[c][0][j0 + j], __fmul_rn(__uint_as_float(r1[j]), inv));
-                run[c][1][j0 + j] = __fadd_rn(run[c][1][j0 + j], __fmul_rn(__uint_as_float(r2[j]), inv));
-              }
-            } else {
-#pragma unroll
-              for (int j = 0; j < 16; ++j) { run[c][0][j0 + j] = __uint_as_float(r1[j]) * inv; run[c][1][j0 + j] = __uint_as_float(r2[j]) * inv; }
+            for (int j = 0; j < 16; ++j) {
+              run[c][0][j0 + j] = __fadd_rn(run[c][0][j0 + j], __fmul_rn(__uint_as_float(r1[j]), inv));
+              run[c][1][j0 + j] = __fadd_rn(run[c][1][j0 + j], __fmul_rn(__uint_as_float(r2[j]), inv));
             }
+          } else {
+#pragma unroll
+            for (int j = 0; j < 16; ++j) { run[c][0][j0 + j] = __uint_as_float(r1[j]) * inv; run[c][1][j0 + j] = __uint_as_float(r2[j]) * inv; }
           }
         }
         tc_fence_before();
@@ -604,56 +578,53 @@ gemm_dense_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant
         }
       }
       if (kEpi == EPI_RESIDUAL) {
-        // EPI_RESIDUAL: the new residual stream, bf16(h * gain), and per 64-feature slot the row's sum of squares in gemm.cu's
-        // order: quads of four features, then a butterfly over the 16 quads (partners 8, 4, 2, 1 apart).  t[e]: the quads of piece e
-        float t[kPieces][8];
+        // EPI_RESIDUAL: the new residual stream, bf16(h * gain), and per 128-feature tile the row's sum of squares in
+        // gemm.cu's order: quads of four features, then a butterfly over the 32 quads (partners 16, 8, 4, 2, 1 apart)
+        float t[kCh][8];
 #pragma unroll
-        for (int e = 0; e < kPieces; ++e) {
-          float(&v)[32] = run[e >> 1][e & 1];
+        for (int c = 0; c < kCh; ++c) {
 #pragma unroll
-          for (int q = 0; q < 8; ++q)
-            t[e][q] = n_base + piece(e) + 4 * q < p.N ? sumsq4(make_float4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3])) : 0.f;
-          const int n = n_base + piece(e) + lc4;
-          const float4 g = n < p.N ? *reinterpret_cast<const float4*>(p.gain + n) : make_float4(0.f, 0.f, 0.f, 0.f);
-          rows_to_buf(trans, lane, v);
+          for (int q = 0; q < 8; ++q) {
+            float part[2] = {0.f, 0.f};
 #pragma unroll
-          for (int i = 0; i < 8; ++i) {
-            const int r = row0 + 4 * i + lr4;
-            const float4 x = *trans_at(trans, 4 * i + lr4, lane & 7);
-            if (ok && r < p.R && n < p.N) {
-              *reinterpret_cast<float4*>(p.h + (size_t)r * p.N + n) = x;
-              *reinterpret_cast<uint2*>(p.hb + (size_t)r * p.N + n) = make_uint2(pack2(x.x * g.x, x.y * g.y), pack2(x.z * g.z, x.w * g.w));
-            }
+            for (int half = 0; half < 2; ++half)
+              if (n_base + col(c) + 64 * half + 4 * q < p.N)
+                part[half] = sumsq4(make_float4(run[c][half][4 * q], run[c][half][4 * q + 1], run[c][half][4 * q + 2], run[c][half][4 * q + 3]));
+            t[c][q] = part[0] + part[1];
           }
-          __syncwarp();
+#pragma unroll
+          for (int half = 0; half < 2; ++half) {
+            const int n = n_base + col(c) + 64 * half + lc4;
+            const float4 g = n < p.N ? *reinterpret_cast<const float4*>(p.gain + n) : make_float4(0.f, 0.f, 0.f, 0.f);
+            rows_to_buf(trans, lane, run[c][half]);
+#pragma unroll
+            for (int i = 0; i < 8; ++i) {
+              const int r = row0 + 4 * i + lr4;
+              const float4 v = *trans_at(trans, 4 * i + lr4, lane & 7);
+              if (ok && r < p.R && n < p.N) {
+                *reinterpret_cast<float4*>(p.h + (size_t)r * p.N + n) = v;
+                *reinterpret_cast<uint2*>(p.hb + (size_t)r * p.N + n) = make_uint2(pack2(v.x * g.x, v.y * g.y), pack2(v.z * g.z, v.w * g.w));
+              }
+            }
+            __syncwarp();
+          }
         }
-        // a slot from its first and second eight quads
-        auto put = [&](int slot, const float (&lo)[8], const float* hi) {
+        float* ex = sSum + ((n_done & 1) * 128 + lrow) * kSumPitch;
+        if (kCh == 1 && group == 1) {
+#pragma unroll
+          for (int q = 0; q < 8; ++q) ex[q] = t[0][q];
+        }
+        if (kCh == 1) epi_bar_sync();
+        if (kCh == 2 || group == 0) {
           float u[8];
 #pragma unroll
-          for (int q = 0; q < 8; ++q) u[q] = lo[q] + hi[q];
+          for (int q = 0; q < 8; ++q) u[q] = t[0][q] + (kCh == 2 ? t[kCh - 1][q] : ex[q]);
 #pragma unroll
           for (int o = 4; o > 0; o >>= 1)
 #pragma unroll
             for (int q = 0; q < o; ++q) u[q] += u[q + o];
-          if (ok && live && slot * 64 < p.N) p.sq_out[(size_t)row * p.sq_out_stride + slot] = u[0];
-        };
-        if constexpr (kFeat == 256) {
-#pragma unroll
-          for (int e = 0; e < 2; ++e) put((n_base + piece(e)) >> 6, t[e], t[e + 2]);        // (pieces 0, 2 and 1, 3: 32 features apart)
-        } else {
-          // group g has the eight quads from 8 g of every slot; the groups complete the slots in turn, each with the other's quads
-          float* ex = sSum + ((n_done & 1) * 128 + lrow) * kSumPitch;
-#pragma unroll
-          for (int e = 0; e < kPieces; ++e)
-            if ((e & 1) != group) {
-#pragma unroll
-              for (int q = 0; q < 8; ++q) ex[8 * e + q] = t[e][q];
-            }
-          epi_bar_sync();
-#pragma unroll
-          for (int e = 0; e < kPieces; ++e)
-            if ((e & 1) == group) put((n_base >> 6) + e, t[e], ex + 8 * e);
+          const int slot = (n_base + (kCh == 2 ? 128 * group : 0)) >> 7;
+          if (ok && live && slot * 128 < p.N) p.sq_out[(size_t)row * p.sq_out_stride + slot] = u[0];
         }
       }
     }
@@ -673,7 +644,7 @@ int launch(cudaStream_t st, const GemmArgs& g, DenseParams p, int sms, int dev) 
   alignas(64) CUtensorMap tmX, tmW;
   const uint64_t w_rows = (uint64_t)gemm_tiles(g.N) * ((g.K + kBlockK - 1) / kBlockK) * 128;
   if (encode_tmap_bf16_2d(&tmX, g.x, (uint64_t)g.R, (uint64_t)g.K, (uint64_t)g.x_pitch, 128) != 0 ||
-      encode_tmap_bf16_2d(&tmW, g.w, w_rows, kBlockK, kBlockK, kFeat == 192 ? 32 : kFeat / 2) != 0)
+      encode_tmap_bf16_2d(&tmW, g.w, w_rows, kBlockK, kBlockK, kFeat / 2) != 0)
     return -4;
   static bool attr_set[kMaxDevices] = {};        // the shared-memory opt-in is per device
   if (!attr_set[dev]) {
@@ -722,25 +693,21 @@ int launch_gemm_dense(cudaStream_t st, const GemmArgs& g) {
     if (cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || n < 2) return -4;
     sm_count[dev] = n;
   }
-  // The width that leaves less of the machine idle in the last wave of tiles.  QKV and gate/up: a 128-feature tile takes 0.6 of the
-  // time of a 256-feature one (three quarters of the bytes, a shorter epilogue; 4096 rows 18.4 / 29.7 and 14.6 / 22.1 us a tile).
-  // EPI_RESIDUAL, in hundredths of a microsecond, of one wave and of four from 512 to 1024 rows: 128 features 780 + 16 a K block and
-  // wave, 192 features 820 + 22, 256 features 1170 + 31.  us, 128 / 192 / 256: d 4096, K 4096 and 12288: 512 rows 18 / 22 / 30 and
-  // 39 / 49 / 67, 768 rows 28 / 23 / 32 and 69 / 52 / 71, 1024 rows 31 / 38 / 35 and 73 / 90 / 74, 4096 rows 121 / 119 / 150 and 306 /
-  // 276 / 276; d 3584, K 18944: 768 rows 101 / 74 / 101.
+  // The width that leaves less of the machine idle in the last wave of tiles.  A 128-feature tile takes 0.6 of the time of a
+  // 256-feature one (three quarters of the bytes, a shorter epilogue): QKV and gate/up at 4096 rows 18.4 / 29.7 and 14.6 /
+  // 22.1 us a tile.  A residual tile adds the exposed part of its epilogue, which is mostly that of the wide one: O 19.5 / 42 us
+  // (64 K blocks), down 47.6 / 78 (192).
   const int sms = sm_count[dev], pairs = sms / 2;
   const long long kb = (g.K + kBlockK - 1) / kBlockK;
-  auto waves = [&](int feat) -> long long { return ((long long)p.m_tiles * ((g.N + feat - 1) / feat) + pairs - 1) / pairs; };
-  if (g.epi == EPI_RESIDUAL) {
-    const long long c128 = 780 + waves(128) * 16 * kb, c192 = 820 + waves(192) * 22 * kb, c256 = 1170 + waves(256) * 31 * kb;
-    if (c192 < c128 && c192 < c256) return launch<192, EPI_RESIDUAL>(st, g, p, sms, dev);
-    return c128 <= c256 ? launch<128, EPI_RESIDUAL>(st, g, p, sms, dev) : launch<256, EPI_RESIDUAL>(st, g, p, sms, dev);
-  }
-  const bool narrow = !(g.epi == EPI_QKV && g.qkv->hd == 64) && waves(128) * 6 < waves(256) * 10;
+  const long long waves256 = ((long long)p.m_tiles * ((g.N + 255) / 256) + pairs - 1) / pairs;
+  const long long waves128 = ((long long)p.m_tiles * ((g.N + 127) / 128) + pairs - 1) / pairs;
+  const bool narrow = g.epi == EPI_RESIDUAL ? waves128 * (60 + 3 * kb) < waves256 * (240 + 4 * kb)
+                                            : !(g.epi == EPI_QKV && g.qkv->hd == 64) && waves128 * 6 < waves256 * 10;
   switch (g.epi) {
     case EPI_LMHEAD: return launch<256, EPI_LMHEAD>(st, g, p, sms, dev);
     case EPI_QKV: return narrow ? launch<128, EPI_QKV>(st, g, p, sms, dev) : launch<256, EPI_QKV>(st, g, p, sms, dev);
-    default: return narrow ? launch<128, EPI_SWIGLU>(st, g, p, sms, dev) : launch<256, EPI_SWIGLU>(st, g, p, sms, dev);
+    case EPI_SWIGLU: return narrow ? launch<128, EPI_SWIGLU>(st, g, p, sms, dev) : launch<256, EPI_SWIGLU>(st, g, p, sms, dev);
+    default: return narrow ? launch<128, EPI_RESIDUAL>(st, g, p, sms, dev) : launch<256, EPI_RESIDUAL>(st, g, p, sms, dev);
   }
 }
 

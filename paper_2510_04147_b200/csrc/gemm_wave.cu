@@ -363,7 +363,7 @@ gemm_wave_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant_
       const int row_end = min(p.R, (2 * mt + crank + 1) * p.half);
       const bool live = row < row_end, any = row0 < row_end;
       float inv = 1.f;
-      if (live) {                            // RMSNorm, consumer side: the producers' sums in slot order
+      if (live) {                            // RMSNorm, consumer side: the producers' per-tile sums in slot order
         const float* q = p.sq + (size_t)row * p.sq_stride;
         float ss = 0.f;
         if (((p.sq_count | p.sq_stride) & 3) == 0) {

@@ -237,7 +237,7 @@ constexpr int kAttnTcMaxNode = 128;     // widest node of the tcgen05 form: its 
 // EPI_RESIDUAL: the split-K CTAs of a tile form a cluster; they sum their accumulators through
 // distributed shared memory in split order, add the residual stream, and write the new stream
 // h (fp32), its bf16 copy times the next norm's gain (hb, the next projection's operand) and the
-// row's sums of squares, one for each 64 features.  The RMSNorm itself is then applied by the consumer:
+// tile's share of every row's sum of squares.  The RMSNorm itself is then applied by the consumer:
 // rmsnorm(h) * g . W^T  ==  inv_rms(row) * ((h * g) . W^T), with inv_rms from the sums of squares.
 // EPI_SUM: the same cluster reduction, the sums themselves go to `out` (fp32 [R][N]).
 // EPI_QKV (dense kernel only): rotary embedding of q and k, everything rounded to bf16; q rows to their buffer, k and v
@@ -292,7 +292,7 @@ struct GemmArgs {
   float* h;              // [R][N] fp32 residual stream, updated in place
   bf16* hb;              // [R][N] bf16(h * gain)
   const float* gain;     // [N]
-  float* sq_out;         // [R][sq_out_stride]: slot s of a row receives the sum of squares of the features [64 s, +64)
+  float* sq_out;         // [R][sq_out_stride]: slot `tile` of a row receives the tile's sum of squares
   int sq_out_stride;
 };
 int gemm_tiles(int N);

@@ -53,7 +53,7 @@ struct ssd_ctx {
   size_t partial_row_floats = 0;   // split-K workspace per row
   float* h = nullptr;
   bf16* xn = nullptr;
-  float* sq = nullptr;           // [R_cap][sq_stride] sums of squares of h, one for each 64 features (fused RMSNorm)
+  float* sq = nullptr;           // [R_cap][sq_stride] per-tile sums of squares of h (fused RMSNorm)
   int sq_stride = 1;
   float* partial = nullptr;
   bf16 *q = nullptr, *att = nullptr, *act = nullptr;
@@ -191,12 +191,13 @@ int capped_split(int s, int k) {
 // tiles against eight (two CTAs per SM), eight layers: 961 / 964 us at 32 rows, 1062 / 1039 at 64, 1267 / 1253 at 128, 1853 / 1740
 // at 256 (half the reads of the activations, half the partial sums to exchange).
 // A power of two: clusters of five leave so many SMs of a GPC unused that 140 CTAs take two waves (28 tiles: 1019 -> 1164 us).
-// Two K blocks each at least: the cluster of the splits shares the rows of the epilogue, which is most of a small launch.  (d 256, ffn
-// 688, forwards of 16 to 80 rows: one split of O's four K blocks and two of down's eleven 82.4 us, two and four 78.6, four and
-// eight 77.6.)
+// Up to four splits may be down to one K block: the cluster of the splits shares the rows of the epilogue, which is most of a small
+// launch.  (d 256, ffn 688: one split of O's four K blocks and two of down's eleven took 91 us a forward of 16 to 80 rows, four
+// of each 86, four and eight 87.)
 int auto_split_residual(int tiles, int k) {
+  const int kb = (k + 63) / 64;
   int s = 8;
-  while (s > 1 && (tiles * s > kSms || 2 * s > (k + 63) / 64)) s >>= 1;
+  while (s > 1 && (tiles * s > kSms || s > kb || (s > 4 && 4 * s > kb))) s >>= 1;
   return s;
 }
 // QKV: its finishing pass reads every split's partial sums.  One CTA per SM against two, eight layers: 36 tiles (4 splits, not 8)
@@ -428,12 +429,8 @@ int forward(ssd_ctx* c, int kind, const int* ids_dev, int R, RowMap map, int n_s
   //   O       17 / 20    20 / 20    21 / 20    25 / 20    28 / 20    30 / 21    42 / 32    45 / 32    49 / 33
   //   gate/up 55 / 61    60 / 55    74 / 90    88 / 92    95 / 93   102 / 86   120 / 130  133 / 130  147 / 126
   //   down    36 / 71    43 / 73    50 / 73    68 / 75    72 / 76    77 / 78   125 / 109  132 / 111  142 / 118
-  // With the loops walked by one lane, pairs in the skinny kernel and 192-feature tiles in the dense one, down (in the live stream):
-  //   rows           288        320        384        416        448        512
-  //   d 4096       34 / 42    38 / 47    48 / 49    56 / 49    61 / 52    - / 52
-  //   d 3584       44 / 62    50 / 69    61 / 70    63 / 68    70 / 71    - / 72
-  // (Where the two shapes disagree - down at 417 to 447 rows, gate/up at 640 - the line costs one of them up to 5 %; other widths
-  // take the same lines unmeasured.)
+  // (Where the two shapes disagree - down at 448 rows, gate/up at 640 - the line costs one of them up to 5 %; other widths take
+  // the same lines unmeasured.)
   const bool may = R > c->dense_rows;
   const bool dense_gu = may && (R <= 256 || R * 16 >= (R + 255) / 256 * 256 * 13);
   const bool dense_qkv = may && (R > 384 || (R <= 256 && gemm_tiles(c->nqkv) >= 74));
@@ -444,7 +441,7 @@ int forward(ssd_ctx* c, int kind, const int* ids_dev, int R, RowMap map, int n_s
   const bool even = R <= 256 && 3 * R > 2 * c->dense_rows;
   const bool even_qkv = even && hd == 128 && gemm_wave_fits(c->nqkv, R, c->split_qkv);
   const bool even_gu = even && gemm_wave_fits(2 * c->ffn_pad, R, 1) && gemm_wave_gains(2 * c->ffn_pad);
-  const bool dense_o = may && R > 256, dense_down = may && R > 416;
+  const bool dense_o = may && R > 256, dense_down = may && R > 448;
   // The attention takes finished (rotated, bf16) q, k and v: the tcgen05 form, and the cache-fill forward, whose K/V go to
   // the cache.  (A function of the node width, never of the number of nodes.)
   const bool bf16_qkv = via_cache || (hd == 128 && c->attn_impl == 1 && map.T <= kAttnTcMaxNode);
@@ -456,7 +453,7 @@ int forward(ssd_ctx* c, int kind, const int* ids_dev, int R, RowMap map, int n_s
     return fail(c, SSD_ERR_OVERFLOW, "attention workspace too small for %d parts x %d rows", n_parts, R);
   const int nl = range.end < 0 ? c->cfg.n_layers : range.end;
   // The RMSNorms have no kernel of their own: a producer (the embedding gather, the O and down
-  // projections) writes the residual stream h, bf16(h * gain) in `xn` and sums of squares (one for each 64 features) in
+  // projections) writes the residual stream h, bf16(h * gain) in `xn` and per-tile sums of squares in
   // `sq`; the consuming projection scales its output rows by 1/rms.
   int sq_count = 1;                       // slots of `sq` the next consumer sums per row
   auto consume_norm = [&](GemmArgs& ga) {
@@ -552,7 +549,7 @@ int forward(ssd_ctx* c, int kind, const int* ids_dev, int R, RowMap map, int n_s
     produce_norm(g, w.g_ffn, c->split_o);
     rc = dense_o ? run_gemm_dense(c, g, SSD_PROF_GEMM_O) : run_gemm(c, g, SSD_PROF_GEMM, SSD_PROF_GEMM_O);
     if (rc) return rc;
-    sq_count = (d + 63) / 64;
+    sq_count = gemm_tiles(d);
     // ---- gate/up projection with SwiGLU
     g = GemmArgs{};
     g.x = c->xn; g.w = w.wgu; g.R = R; g.N = 2 * c->ffn_pad; g.K = d; g.x_pitch = d; g.w_pitch = d; g.w_tiled = 1;
@@ -814,7 +811,7 @@ int ssd_create(const ssd_config* cfg, void* cuda_stream, ssd_ctx** out) {
     const size_t R = (size_t)c->R_cap;
     ALLOC(c, c->h, R * d);
     ALLOC(c, c->xn, R * d);
-    c->sq_stride = (d + 63) / 64;
+    c->sq_stride = gemm_tiles(d);
     ALLOC(c, c->sq, R * c->sq_stride);
     c->partial_row_floats = (size_t)kMaxSplit * d;
     if ((size_t)4 * c->nqkv > c->partial_row_floats) c->partial_row_floats = (size_t)4 * c->nqkv;
