@@ -7,7 +7,7 @@
 // (each CTA stages its own 128 rows and half of the features; 32 KB or less per 64-wide K block, six or seven stages
 // deep).  The accumulator has rows in the lanes and features in the columns, so an epilogue thread owns part of a row:
 // the RMSNorm scale, the rotary pairs, SwiGLU's gate and up all sit in one thread and no transpose is needed.  The
-// accumulators (two of 256 or 192 columns, four of 128) fill the tensor memory: the epilogue of a tile runs under the main
+// accumulators (two of 256 columns or four of 128) fill the tensor memory: the epilogue of a tile runs under the main
 // loop of the next.  Tiles are walked rows first, so that the CTAs in flight share a few weight tiles and all of the
 // activations through L2.
 //
