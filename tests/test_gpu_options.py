@@ -1,0 +1,27 @@
+"""Options at the ends of what they accept: the value that stands for "never"."""
+import numpy as np
+import pytest
+
+from paper_2510_04147_b200 import workloads as wl
+
+pytestmark = pytest.mark.gpu
+
+
+def test_the_largest_dense_rows_means_never():
+    from paper_2510_04147_b200 import binding
+    w = wl.TINY.replace(name="options", n_layers=1, vocab=512, n_heads=2, n_kv_heads=2, head_dim=128, prompt_len=40, gen_len=16)
+    ids = np.arange(16, dtype=np.int32)[None, None]
+    ssd = binding.Ssd(binding.config_from_workload(w, max_drafts=0))
+    try:
+        ssd.load_workload_weights(w)
+        ssd.prefill(wl.make_prompts(w).numpy())
+        launches = []
+        for dense_rows in (1 << 20, (1 << 30) - 1, 1 << 30, 2**31 - 1, 0):
+            ssd.set_option("dense_rows", dense_rows)
+            before = ssd.launch_count()
+            ssd.verify_forward(ids, np.ones((1, 1, 16), np.uint8))
+            launches.append(ssd.launch_count() - before)
+        # (the evenly shared q|k|v projection needs no pass that finishes q, k and v)
+        assert len(set(launches[:-1])) == 1 and launches[-1] < launches[0], launches
+    finally:
+        ssd.destroy()
