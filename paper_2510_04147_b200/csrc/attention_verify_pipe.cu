@@ -491,7 +491,8 @@ attn_verify_pipe_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
         __syncwarp();
         if (lane == 0) mbar_arrive(bar_sfree0 + 8u * (uint32_t)((u - 1) & 1));
       }
-      ok = mbar_wait(bar_s0 + 8u * (uint32_t)(u & 1), (uint32_t)((u >> 1) & 1), abort_flag);
+      // (here and below: a wait that expired is never forgotten, whatever a later one says - the error word depends on it)
+      ok = ok && mbar_wait(bar_s0 + 8u * (uint32_t)(u & 1), (uint32_t)((u >> 1) & 1), abort_flag);
       tc_fence_after();
       ok = __all_sync(0xffffffffu, ok ? 1 : 0) != 0;        // the tensor-memory accesses below are warp-wide
       const uint32_t tmem_S = tmem_base + (uint32_t)(u & 1) * 128u;
@@ -536,7 +537,7 @@ attn_verify_pipe_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
       if (kShared && u > 0) l_row = l_row * corr_prev + tile_sum(u - 1);      // (every chunk sum of the previous tile is visible now)
       if (kShared && u == fresh_at) {                   // this tile starts a part: put the one before away
         fresh_at = g.begin(++next_part) - first;
-        ok = mbar_wait(bar_o0 + 8u * (uint32_t)((u - 1) & 1), (uint32_t)(((u - 1) >> 1) & 1), abort_flag);
+        ok = ok && mbar_wait(bar_o0 + 8u * (uint32_t)((u - 1) & 1), (uint32_t)(((u - 1) >> 1) & 1), abort_flag);
         tc_fence_after();
         ok = __all_sync(0xffffffffu, ok ? 1 : 0) != 0;
         if (ok) part_done(m_row, l_row);
@@ -556,7 +557,7 @@ attn_verify_pipe_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
       // tensor memory, where tiles alternate) the one before
       const int must = (rescale || !kTmemP) ? u - 1 : u - 2;
       if (must >= 0) {
-        ok = mbar_wait(bar_o0 + 8u * (uint32_t)(must & 1), (uint32_t)((must >> 1) & 1), abort_flag);
+        ok = ok && mbar_wait(bar_o0 + 8u * (uint32_t)(must & 1), (uint32_t)((must >> 1) & 1), abort_flag);
         tc_fence_after();
         ok = __all_sync(0xffffffffu, ok ? 1 : 0) != 0;
       }
@@ -623,11 +624,9 @@ attn_verify_pipe_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
       m_row = m_new;
     }
     if (!broke) ok = softmax_barrier_and(ok);               // the last tile's chunk sums are visible
-    if (ok) {
-      l_row = l_row * corr_prev + tile_sum(n_tiles - 1);
-      ok = mbar_wait(bar_o0 + 8u * (uint32_t)((n_tiles - 1) & 1), (uint32_t)(((n_tiles - 1) >> 1) & 1), abort_flag);
-      tc_fence_after();
-    }
+    if (ok) l_row = l_row * corr_prev + tile_sum(n_tiles - 1);
+    ok = ok && mbar_wait(bar_o0 + 8u * (uint32_t)((n_tiles - 1) & 1), (uint32_t)(((n_tiles - 1) >> 1) & 1), abort_flag);
+    tc_fence_after();
     ok = __all_sync(0xffffffffu, ok ? 1 : 0) != 0;
     // this CTA's last part; a CTA that has not the first part of all hands two parts on as two entries
     const bool two = kShared && have && rank > 0;
