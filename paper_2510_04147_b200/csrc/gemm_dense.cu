@@ -418,8 +418,8 @@ gemm_dense_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant
           float x[32];
 #pragma unroll
           for (int j = 0; j < 16; ++j) {
-            x[j] = p.sq != nullptr ? __uint_as_float(r1[j]) * inv : __uint_as_float(r1[j]);
-            x[16 + j] = p.sq != nullptr ? __uint_as_float(r2[j]) * inv : __uint_as_float(r2[j]);
+            x[j] = p.sq != nullptr ? __fmul_rn(__uint_as_float(r1[j]), inv) : __uint_as_float(r1[j]);
+            x[16 + j] = p.sq != nullptr ? __fmul_rn(__uint_as_float(r2[j]), inv) : __uint_as_float(r2[j]);
           }
           if (some_dead) {
 #pragma unroll

@@ -318,7 +318,8 @@ int encode_tmap_bf16_2d(void* map_out, const void* base, uint64_t rows, uint64_t
 #ifdef __CUDACC__
 // ---- what the LM head keeps of a vocabulary tile of 128 entries, per row: maximum with the lowest index among equals, sum of
 // exp(x - its maximum) and, where asked, the largest entries.  A tile is worked on in quarters of 32 entries, merged (0 + 1) + (2 + 3),
-// in every kernel and whoever has the quarters: the value depends on the tile alone.
+// in every kernel and whoever has the quarters; every rounding is spelled out, so the value depends on the tile alone, not on what a
+// compiler contracts where the entries come from a product in registers.
 struct LmStat { float m, sum; int arg; };
 __device__ __forceinline__ LmStat lm_quarter(const float (&x)[32], int first) {
   LmStat s{-INFINITY, 0.f, 0x7fffffff};
@@ -327,15 +328,15 @@ __device__ __forceinline__ LmStat lm_quarter(const float (&x)[32], int first) {
     if (x[j] > s.m) { s.m = x[j]; s.arg = first + j; }
   if (s.m != -INFINITY) {
 #pragma unroll
-    for (int j = 0; j < 32; ++j) s.sum = __fadd_rn(s.sum, expf(x[j] - s.m));              // (exp(-inf) = 0 for dead entries)
+    for (int j = 0; j < 32; ++j) s.sum = __fadd_rn(s.sum, expf(__fsub_rn(x[j], s.m)));    // (exp(-inf) = 0 for dead entries)
   }
   return s;
 }
 // the same value from both partners: the lower quarter's (maximum, index) wins a tie
 __device__ __forceinline__ LmStat lm_merge(const LmStat& lo, const LmStat& hi) {
   LmStat s{fmaxf(lo.m, hi.m), 0.f, hi.m > lo.m ? hi.arg : lo.arg};
-  if (lo.m != -INFINITY) s.sum = __fmaf_rn(lo.sum, expf(lo.m - s.m), s.sum);
-  if (hi.m != -INFINITY) s.sum = __fmaf_rn(hi.sum, expf(hi.m - s.m), s.sum);
+  if (lo.m != -INFINITY) s.sum = __fmaf_rn(lo.sum, expf(__fsub_rn(lo.m, s.m)), s.sum);
+  if (hi.m != -INFINITY) s.sum = __fmaf_rn(hi.sum, expf(__fsub_rn(hi.m, s.m)), s.sum);
   return s;
 }
 // sorted lists (value descending, lower index first): an insertion only where an entry beats the last of the list
