@@ -312,9 +312,10 @@ int ssd_profile_read(ssd_ctx* ctx, int64_t* launches, double* milliseconds, doub
  *   "attn_impl"  1 = attention of the verification forward on tcgen05 where the shape allows (head
  *        dimension 128, nodes of up to 128 rows), the default; 0 = always the mma.sync form;
  *   "attn_pipe_ctas", "attn_pipe_keys" with attn_impl 1: a prefilled batch that gives at least attn_pipe_ctas
- *        (default 64, from 1024 cached keys on 75) pairs (head, sequence) - batch * heads - has one CTA per pair walk all key
- *        tiles, instead of cutting them into parts that a cluster can share; one sequence is faster with its key parts side by
- *        side.  attn_pipe_keys (default 1; 0 = never) is the shortest prefix that may take it.
+ *        pairs (head, sequence) - batch * heads - has one CTA per pair walk all key tiles, instead of cutting them into parts
+ *        that a cluster can share; one sequence is faster with its key parts side by side.  The default, 64, stands for 75 from
+ *        1024 cached keys on; every other value is the line for all prefixes.  attn_pipe_keys (default 1; 0 = never) is the
+ *        shortest prefix that may take it.
  *        The two forms sum in different orders, so a sequence's bits depend on the prefilled batch SIZE - never
  *        on the other sequences' contents, on the node count, or on which sequences are still unfinished;
  *   "dense_rows" in forwards of more rows than this (default 240) a projection may run as a dense contraction instead

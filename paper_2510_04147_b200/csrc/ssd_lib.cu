@@ -25,6 +25,7 @@ struct LayerW {
 struct ProfRec { int fam, sub; cudaEvent_t e0, e1; double bytes; };
 struct MarkRec { int fam, sub; double bytes; };
 constexpr int kMaxMarks = 16384;      // launches one in-stream measurement can hold
+constexpr int kPipeCtas = 64;         // default of "attn_pipe_ctas"; stands for 75 from 1024 keys on (pipe_parts)
 
 char g_create_error[256] = "";
 
@@ -119,7 +120,7 @@ struct ssd_ctx {
   int64_t launches = 0;
   int gemm_max_stages = 0;       // tuning: cap on the projection kernel's ring depth (0: none)
   int attn_pipe_keys = 1;        // prefixes of at least this many keys take the pipelined attention form (0: never) ...
-  int attn_pipe_ctas = 0;        // ... when the prefilled batch gives it at least this many (head, sequence) CTAs (0: pipe_parts' own line)
+  int attn_pipe_ctas = kPipeCtas;          // ... when the prefilled batch gives it at least this many (head, sequence) CTAs
   int wait_limit_us = 0;         // bound of the projection kernel's barrier waits (0: the kernel's default, 2 s)
   int starve_gemm_kb = 0;        // test hook for ssd_gemm_bf16: K block (1-based) whose copies are left out
   bool profiling = false;        // mode 1: CUDA events around every launch (serialises the stream)
@@ -225,7 +226,7 @@ int kv_split_for(const ssd_ctx* c, int S) {
 // parts, us of four layers at 64 and 256 rows: 512 keys 607 / 612 and 954 / 952, 1024 keys 625 / 622 and 978 / 964, 2048 keys
 // 662 / 641 and 1045 / 992, 4096 keys 755 / 699 and 1163 / 1042.
 int pipe_parts(const ssd_ctx* c, int S) {
-  const int one_from = c->attn_pipe_ctas > 0 ? c->attn_pipe_ctas : (S >= 1024 ? kSms / 2 + 1 : 64);
+  const int one_from = c->attn_pipe_ctas == kPipeCtas && S >= 1024 ? kSms / 2 + 1 : c->attn_pipe_ctas;
   if (c->attn_pipe_keys > 0 && S >= c->attn_pipe_keys && c->batch * c->H >= one_from) return 1;
   int n = c->kv_split_opt > 0 ? (S + c->kv_split_opt - 1) / c->kv_split_opt + 1 : (c->H <= 16 ? 8 : (c->H <= 32 ? 4 : 2));
   return std::min(std::max(n, 2), kAttnMaxClusterParts);
