@@ -413,7 +413,7 @@ attn_fill_tc_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_consta
 template <int kQ>
 int launch(cudaStream_t st, const AttnArgs& a, const CUtensorMap& tmQ, const CUtensorMap& tmK, const CUtensorMap& tmV) {
   const size_t smem = (size_t)(kQ + 2 * kStages) * kTileBytes + 1024 + 256;
-  static bool attr_set[kMaxDevices] = {};          // the shared-memory opt-in is per device
+  static PerDevice<bool> attr_set = {};             // the shared-memory opt-in
   const int dev = device_slot();
   if (dev < 0) return -4;
   if (!attr_set[dev]) {

@@ -515,7 +515,7 @@ int launch_attention_verify(cudaStream_t st, const AttnArgs& a) {
   // two CTAs per SM by default; three (register-capped build) when only that keeps the grid in one wave
   const long long n_ctas = (long long)a.n_seq_slots * q_tiles * n_parts * a.H;
   const bool dense = qt_rows == 32 && n_ctas > 2 * kSms;
-  static bool attr_set[kMaxDevices] = {};        // the shared-memory opt-in is per device
+  static PerDevice<bool> attr_set = {};             // the shared-memory opt-in
   const int dev = device_slot();
   if (dev < 0) return -4;
   if (!attr_set[dev]) {

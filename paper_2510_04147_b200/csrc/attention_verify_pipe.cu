@@ -45,8 +45,6 @@
 #include <cuda.h>
 #include <string.h>
 
-#include <atomic>
-
 namespace ssd {
 
 namespace {
@@ -721,7 +719,7 @@ attn_verify_pipe_kernel(const __grid_constant__ CUtensorMap tmQ, const __grid_co
 template <int QT, bool kShared>
 cudaError_t launch_pipe(cudaStream_t st, dim3 grid, size_t smem, const CUtensorMap (&tm)[5], const AttnArgs& a, const PipeShape& g,
                         float scale_log2) {
-  static std::atomic<bool> attr_set[kMaxDevices] = {};        // the shared-memory opt-in is per device
+  static PerDevice<bool> attr_set = {};             // the shared-memory opt-in
   const int dev = device_slot();
   if (dev < 0) return cudaErrorInvalidDevice;
   if (!attr_set[dev]) {

@@ -21,8 +21,6 @@
 #include <math.h>
 #include <stdio.h>
 
-#include <atomic>
-
 namespace ssd {
 
 int gemm_tiles(int N) { return (N + 127) / 128; }
@@ -818,7 +816,7 @@ int launch_gemm_tc(cudaStream_t st, const GemmArgs& g) {
   }
   if (!make_tmap(&tmX, g.x, (uint64_t)g.R, (uint64_t)g.K, (uint64_t)g.x_pitch, (uint32_t)(p.two_sm ? p.npad / 2 : p.npad))) return -4;
   // the opt-in to more than 48 KB of dynamic shared memory is a per-device attribute of the function
-  static std::atomic<bool> smem_set[kMaxDevices] = {};
+  static PerDevice<bool> smem_set = {};
   const int dev = device_slot();
   if (dev < 0) return -4;
   if (!smem_set[dev]) {

@@ -646,7 +646,7 @@ int launch(cudaStream_t st, const GemmArgs& g, DenseParams p, int sms, int dev) 
   if (encode_tmap_bf16_2d(&tmX, g.x, (uint64_t)g.R, (uint64_t)g.K, (uint64_t)g.x_pitch, 128) != 0 ||
       encode_tmap_bf16_2d(&tmW, g.w, w_rows, kBlockK, kBlockK, kFeat / 2) != 0)
     return -4;
-  static bool attr_set[kMaxDevices] = {};        // the shared-memory opt-in is per device
+  static PerDevice<bool> attr_set = {};             // the shared-memory opt-in
   if (!attr_set[dev]) {
     if (cudaFuncSetAttribute(gemm_dense_kernel<kFeat, kEpi>, cudaFuncAttributeMaxDynamicSharedMemorySize, Cfg<kFeat>::kSmem) != cudaSuccess) return -4;
     attr_set[dev] = true;
@@ -685,7 +685,7 @@ int launch_gemm_dense(cudaStream_t st, const GemmArgs& g) {
   if (g.qkv) p.qkv = *g.qkv;
   p.tile_max = g.tile_max; p.tile_sum = g.tile_sum; p.tile_arg = g.tile_arg; p.topk = g.topk; p.tile_topv = g.tile_topv; p.tile_topi = g.tile_topi;
   p.mask_id = g.mask_id;
-  static int sm_count[kMaxDevices] = {};
+  static PerDevice<int> sm_count = {};
   const int dev = device_slot();
   if (dev < 0) return -4;
   if (sm_count[dev] == 0) {

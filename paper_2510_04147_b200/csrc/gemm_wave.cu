@@ -529,7 +529,7 @@ int launch(cudaStream_t st, const GemmArgs& g, WaveParams p, int dev) {
   if (encode_tmap_bf16_2d(&tmX, g.x, (uint64_t)g.R, (uint64_t)g.K, (uint64_t)g.x_pitch, (uint32_t)p.half) != 0) return -4;
   for (int i = 0; i < 4; ++i)
     if (encode_tmap_bf16_2d(&tmW.by_rows[i], g.w, w_rows, kBlockK, kBlockK, 64u >> i) != 0) return -4;
-  static bool attr_set[kMaxDevices] = {};        // the shared-memory opt-in is per device
+  static PerDevice<bool> attr_set = {};             // the shared-memory opt-in
   if (!attr_set[dev]) {
     if (cudaFuncSetAttribute(gemm_wave_kernel<kEpi, kWide>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemMax) != cudaSuccess) return -4;
     attr_set[dev] = true;

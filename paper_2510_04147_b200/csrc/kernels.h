@@ -5,6 +5,8 @@
 #include <stddef.h>
 #include <stdint.h>
 
+#include <atomic>
+
 typedef __nv_bfloat16 bf16;
 
 namespace ssd {
@@ -117,8 +119,11 @@ constexpr int kSms = 148;
 
 // ---------------------------------------------------------------- per-device set-up
 // Function attributes (the opt-in to large dynamic shared memory) belong to a device, not to the
-// process: launchers keep one flag per device ordinal and set the attribute on a device's first use.
+// process: launchers keep one flag per device ordinal and set the attribute on a device's first use, which threads with a
+// context each may reach together (then each of them sets it).
 constexpr int kMaxDevices = 64;
+template <typename T>
+using PerDevice = std::atomic<T>[kMaxDevices];
 inline int device_slot() {
   int dev = -1;
   if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDevices) return -1;
