@@ -320,8 +320,8 @@ int ssd_profile_read(ssd_ctx* ctx, int64_t* launches, double* milliseconds, doub
  *        on the other sequences' contents, on the node count, or on which sequences are still unfinished;
  *   "dense_rows" in forwards of more rows than this (default 240) a projection may run as a dense contraction instead
  *        of a stream of the weights, and from two thirds of it on the LM head likewise and (up to 256 rows) a projection with its
- *        features shared out evenly over the SMs, where its size makes that the faster one; the results are bit-identical
- *        either way;
+ *        features shared out evenly over the SMs, where its size makes that the faster one (0: wherever they can run, whatever
+ *        the size); the results are bit-identical either way;
  *   "two_sm_rows" the QKV, gate/up and LM-head projections, and O and down where their clusters find room, run pairs of weight
  *        tiles as ONE tcgen05.mma with cta_group::2 (two CTAs, M = 256, each SM holding half of the activation tile)
  *        from this many padded rows per launch on; 0 = never; default 128, where it starts to pay.  The results

@@ -7,6 +7,8 @@
 
 #include <atomic>
 
+#include "routes.h"
+
 typedef __nv_bfloat16 bf16;
 
 namespace ssd {
@@ -112,10 +114,6 @@ inline cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, s
   return launch_pdl_cluster_xy(kernel, grid, block, smem, st, 1u, 1u, true, args...);
 }
 #endif
-
-// The rules that share work out are functions of the shape alone, so they take the machine's size from here; a grid of
-// persistent CTAs asks the device.
-constexpr int kSms = 148;
 
 // ---------------------------------------------------------------- per-device set-up
 // Function attributes (the opt-in to large dynamic shared memory) belong to a device, not to the

@@ -440,9 +440,10 @@ int forward(ssd_ctx* c, int kind, const int* ids_dev, int R, RowMap map, int n_s
   // 160 1420 / 1410 / 1422, 192 1545 / 1533 / 1499, 224 1742 / 1692 / 1660, 256 1766 / 1696 / 1705; d 3584, ffn 18944 (36 tiles of
   // four splits; 296 tiles go evenly as they are): 128 rows 1307 / 1300 / 1343, 192 1596 / 1575 / 1613, 256 1773 / 1738 / 1783.
   const bool two_thirds = 3LL * R > 2LL * c->dense_rows;      // (the option may be any int: a very large one means never)
+  const bool anywhere = c->dense_rows == 0;                   // (0: wherever these kernels can run, not only where they are the faster ones)
   const bool even = R <= 256 && two_thirds;
   const bool even_qkv = even && hd == 128 && gemm_wave_fits(c->nqkv, R, c->split_qkv);
-  const bool even_gu = even && gemm_wave_fits(2 * c->ffn_pad, R, 1) && gemm_wave_gains(2 * c->ffn_pad);
+  const bool even_gu = even && gemm_wave_fits(2 * c->ffn_pad, R, 1) && (anywhere || gemm_wave_gains(2 * c->ffn_pad));
   const bool dense_o = may && R > 256, dense_down = may && R > 448;
   // The attention takes finished (rotated, bf16) q, k and v: the tcgen05 form, and the cache-fill forward, whose K/V go to
   // the cache.  (A function of the node width, never of the number of nodes.)
@@ -592,10 +593,9 @@ int forward(ssd_ctx* c, int kind, const int* ids_dev, int R, RowMap map, int n_s
     } else {
       g.epi = EPI_LMHEAD; g.tile_max = c->tile_max; g.tile_sum = c->tile_sum; g.tile_arg = c->tile_arg;
       if (range.topk > 0) { g.topk = range.topk; g.tile_topv = c->tile_topv; g.tile_topi = c->tile_topi; }
-      // The dense kernel has the statistics of a tile under the next one's main loop; where its 256-row tiles are filled.  us,
-      // skinny / dense, V 126464, d 4096: 32 rows 164 / 192, 128 rows 202 / 202, 160 223 / 211, 192 246 / 220, 256 287 / 228, 320
-      // 350 / 385, 512 497 / 402; V 152064, d 3584: 128 rows 221 / 233, 256 288 / 252, 320 395 / 418.
-      const bool dense_lm = two_thirds && (R <= 256 || R * 16 >= (R + 255) / 256 * 256 * 13);
+      // Where the dense kernel's 256-row tiles are filled and its turns are the shorter ones.  us, skinny / dense, V 126464, d 4096: 32
+      // rows 164 / 192, 128 rows 202 / 202, 320 350 / 385; V 152064, d 3584: 128 rows 221 / 233, 320 395 / 418.
+      const bool dense_lm = two_thirds && (R <= 256 || R * 16 >= (R + 255) / 256 * 256 * 13) && (anywhere || lm_head_dense(c->V, d, R));
       int rc = dense_lm ? run_gemm_dense(c, g, -1, SSD_PROF_LMHEAD) : run_gemm(c, g, SSD_PROF_LMHEAD);
       if (rc) return rc;
       Scope sc(c, SSD_PROF_LMHEAD, (double)gemm_tiles(c->V) * R * 12.0, range.topk > 0 ? 2 : 1);

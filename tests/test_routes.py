@@ -1,0 +1,45 @@
+"""The rules by which a call takes one kernel or another, held against what both sides took on a B200 (us, the same process and minute)."""
+import subprocess
+
+import pytest
+
+from paper_2510_04147_b200 import build
+
+
+@pytest.fixture(scope="module")
+def rule(tmp_path_factory):
+    """rule(expressions): their values, as the host code has them."""
+    folder = tmp_path_factory.mktemp("routes")
+
+    def values(expressions):
+        (folder / "r.cpp").write_text('#include "routes.h"\n#include <cstdio>\nusing namespace ssd;\nint main() {\n' +
+                                      "".join(f'std::printf("%d\\n", (int)({e}));\n' for e in expressions) + "}\n")
+        r = subprocess.run(["g++", "-std=c++17", "-I", build.CSRC, "-o", str(folder / "r"), str(folder / "r.cpp")], capture_output=True, text=True)
+        assert r.returncode == 0, r.stderr
+        return [int(x) for x in subprocess.run([str(folder / "r")], capture_output=True, text=True, check=True).stdout.split()]
+    return values
+
+
+def within(took, best):
+    return took <= 1.05 * best + 0.5          # what runs of one side differ by
+
+
+# (vocabulary, d, rows): skinny, dense; LM head and merge kernel, behind other layers
+LM_HEAD = {
+    (512, 256, 192): (15.4, 14.5), (2048, 256, 192): (15.8, 15.0), (2048, 256, 256): (18.7, 15.0), (2048, 256, 512): (19.1, 15.8),
+    (8192, 256, 256): (19.2, 15.4), (2048, 512, 192): (16.7, 16.3), (2048, 512, 256): (19.7, 16.7), (2048, 512, 512): (20.6, 17.4),
+    (24576, 256, 192): (21.2, 25.4), (65536, 256, 192): (41.2, 50.1), (100352, 256, 192): (58.2, 66.9), (128256, 256, 256): (93.5, 79.8),
+    (16384, 512, 192): (18.3, 22.3), (32000, 512, 192): (28.7, 33.2), (65536, 512, 256): (60.2, 52.3), (128256, 512, 512): (180.1, 125.7),
+    (512, 1024, 192): (18.3, 30.9), (2048, 1024, 224): (21.4, 27.1), (16384, 1024, 512): (35.1, 39.5), (24576, 1024, 192): (28.5, 39.8),
+    (32000, 1024, 256): (38.6, 42.1), (50304, 1024, 256): (63.8, 55.0), (65536, 1024, 192): (59.0, 64.8), (65536, 1024, 448): (111.4, 81.1),
+    (2048, 2048, 192): (22.0, 28.4), (16384, 2048, 192): (26.5, 32.9), (50304, 2048, 192): (75.3, 60.0), (128256, 2048, 192): (147.6, 131.8),
+    (2048, 4096, 192): (30.3, 39.4), (8192, 4096, 416): (36.3, 41.4), (16384, 4096, 192): (40.2, 44.6), (50304, 4096, 192): (126.4, 93.2),
+    (128256, 4096, 192): (245.7, 214.2), (128256, 4096, 512): (479.3, 399.4), (126464, 4096, 161): (223.0, 211.0), (152064, 3584, 256): (288.0, 252.0),
+}
+
+
+def test_lm_head_takes_no_slower_kernel(rule):
+    took = rule([f"lm_head_dense({v}, {k}, {r})" for v, k, r in LM_HEAD])
+    for (case, times), dense in zip(LM_HEAD.items(), took):
+        assert within(times[dense], times[0]), (case, dense)
+    assert within(sum(t[d] for t, d in zip(LM_HEAD.values(), took)), sum(min(t) for t in LM_HEAD.values()))
