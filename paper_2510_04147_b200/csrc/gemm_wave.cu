@@ -42,7 +42,6 @@ template <int kEpi> constexpr int kEpiWarpEnd = 2 + kEpiThreads<kEpi> / 32;
 template <int kEpi> constexpr int kTransWarp = kEpi == EPI_SWIGLU ? 32 * 32 : 32 * 128;
 template <int kEpi> constexpr int kTransBytes = kEpiThreads<kEpi> / 32 * kTransWarp<kEpi>;
 constexpr int kMaxStages = 20, kMaxBufs = 4, kMaxBoxes = 12;
-constexpr int kMaxCouples = 256;
 constexpr int kBarBytes = 512, kListBytes = kProducers * kMaxBoxes * 16;
 constexpr int kSmemMax = 226 * 1024;
 constexpr unsigned long long kWaitLimitNs = 2000000000ull;
@@ -540,22 +539,13 @@ int launch(cudaStream_t st, const GemmArgs& g, WaveParams p, int dev) {
   return launch_pdl_cluster(gemm_wave_kernel<kEpi, kWide>, grid, dim3(kThreads<kEpi>), (size_t)smem, st, 2u, tmX, tmW, p) == cudaSuccess ? 0 : -4;
 }
 
-// Couples of a unit: in as few turns as the width of an accumulator allows, one unit for every pair of SMs in each.
-int couples_of_unit(int N, int m_tiles) {
-  const long long work = (long long)(N / 2) * m_tiles, pairs = kSms / 2;
-  for (int turns = 1;; ++turns) {
-    const long long cpu = ((work + pairs * turns - 1) / (pairs * turns) + 7) & ~7ll;
-    if (cpu <= kMaxCouples) return cpu < 16 ? 16 : (int)cpu;
-  }
-}
 int unit_columns(int cpu) { return 2 * ((cpu + 15) & ~15); }
 
 }  // namespace
 
 bool gemm_wave_fits(int N, int R, int splits) {
-  return N % 128 == 0 && splits * unit_columns(couples_of_unit(N, (R + 255) / 256)) <= 512;
+  return N % 128 == 0 && splits * unit_columns(wave_share(N, (R + 255) / 256).couples) <= 512;
 }
-bool gemm_wave_gains(int N) { return (gemm_tiles(N) + kSms - 1) / kSms * 128 * 4 >= couples_of_unit(N, 1) * 5; }
 
 int launch_gemm_wave(cudaStream_t st, const GemmArgs& g) {
   if ((g.x_pitch % 8) || (((uintptr_t)g.x) & 15) || (((uintptr_t)g.w) & 15) || !g.w_tiled || !g.sq || g.sq_count < 1 || g.norm_dim < 1) return -2;
@@ -567,7 +557,7 @@ int launch_gemm_wave(cudaStream_t st, const GemmArgs& g) {
   p.half = ((g.R + 2 * p.m_tiles - 1) / (2 * p.m_tiles) + 7) & ~7;
   const int dev = device_slot();
   if (dev < 0) return -4;
-  p.cpu = couples_of_unit(g.N, p.m_tiles);
+  p.cpu = wave_share(g.N, p.m_tiles).couples;
   p.units = (p.couples + p.cpu - 1) / p.cpu;
   const int cols = unit_columns(p.cpu);
   p.n0 = p.cpu < 128 ? cols : 256;

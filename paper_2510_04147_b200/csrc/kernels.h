@@ -307,7 +307,6 @@ int launch_gemm_dense(cudaStream_t st, const GemmArgs& g);
 // EPI_SWIGLU.  The same sums as the other kernels with the same splits.  Returns 0 or a negative ssd error code.
 int launch_gemm_wave(cudaStream_t st, const GemmArgs& g);
 bool gemm_wave_fits(int N, int R, int splits);     // its accumulators have room for the K splits
-bool gemm_wave_gains(int N);                       // an SM has a fifth less to do than in turns of whole tiles (up to 256 rows)
 // tensor-core path (TMA + tcgen05). Returns 0 or a negative ssd error code.
 int launch_gemm_tc(cudaStream_t st, const GemmArgs& g);
 int gemm_tc_init();   // resolves the driver entry point for tensor-map encoding

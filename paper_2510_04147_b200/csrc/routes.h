@@ -28,4 +28,32 @@ inline bool lm_head_dense(int V, int K, int R) {
   return turns >= 2 && 97 * ceil_div(tiles, pairs) <= turns * block_rows;
 }
 
+// Evenly shared projections (gemm_wave.cu): the couples of a feature and its partner that make a unit, in as few turns as the width of an
+// accumulator allows, one unit for every pair of SMs in each.
+struct WaveShare { int turns, couples; };
+inline WaveShare wave_share(int N, int m_tiles) {
+  const long long work = (long long)(N / 2) * m_tiles, pairs = kSms / 2;
+  for (int turns = 1;; ++turns) {
+    const long long couples = (ceil_div(work, pairs * turns) + 7) & ~7;
+    if (couples <= 256) return {turns, couples < 16 ? 16 : (int)couples};
+  }
+}
+
+// Gate|up shared out evenly instead of in whole tiles (up to 256 rows): the features an SM has to do, in all turns of either.
+// `dense`: the other kernel is the dense one, 256 features to a pair of SMs in a turn; else the skinny one, two tiles of 128 to an SM
+// (one, where there are no more tiles than SMs).  One turn pays from a fifth less on, several, which have no other unit's
+// main loop over their epilogue, from a ninth.  us, other / even, 192 rows and (dense) 256 rows, d 4096 unless said:
+//   features 24576 (256 / 168)   47 / 39, 48 / 41      38912 (512 / 272 and 384 / 272)  88 / 68, 81 / 73
+//   28672 (256 / 200)            50 / 47, 54 / 48      49152 (512 / 336, 384 / 336)     96 / 80, 83 / 83;  d 2048 52 / 42, 42 / 45
+//   37888 (256 / 256)            57 / 57, 58 / 61      53248 (512 / 368, 384 / 368)     103 / 88, 86 / 90
+//   1408, d 256 (128 / 16)       7.6 / 5.3, 6.7 / 5.4  67584 (512 / 464)                115 / 115, 115 / 110 (a forward of four layers 1049 / 1058, 1058 / 1093)
+//   65536 (512 / 448)            112 / 105, 115 / 109  75776 (512 / 512)                121 / 121, 117 / 125
+//   76800 (768 / 528, 640 / 528) 155 / 125, 146 / 134  90112, d 2048 (768 / 624, 640 / 624)  86 / 73, 67 / 74
+inline bool gemm_wave_gains(int N, bool dense) {
+  const int tiles = ceil_div(N, 128);
+  const int other = dense ? ceil_div(ceil_div(N, 256), kSms / 2) * 128 : tiles <= kSms ? 128 : ceil_div(tiles, 2 * kSms) * 256;
+  const WaveShare share = wave_share(N, 1);
+  return share.turns == 1 ? 4 * other >= 5 * share.couples : 8LL * other >= 9LL * share.turns * share.couples;
+}
+
 }  // namespace ssd

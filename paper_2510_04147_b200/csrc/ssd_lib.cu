@@ -443,7 +443,7 @@ int forward(ssd_ctx* c, int kind, const int* ids_dev, int R, RowMap map, int n_s
   const bool anywhere = c->dense_rows == 0;                   // (0: wherever these kernels can run, not only where they are the faster ones)
   const bool even = R <= 256 && two_thirds;
   const bool even_qkv = even && hd == 128 && gemm_wave_fits(c->nqkv, R, c->split_qkv);
-  const bool even_gu = even && gemm_wave_fits(2 * c->ffn_pad, R, 1) && (anywhere || gemm_wave_gains(2 * c->ffn_pad));
+  const bool even_gu = even && gemm_wave_fits(2 * c->ffn_pad, R, 1) && (anywhere || gemm_wave_gains(2 * c->ffn_pad, dense_gu));
   const bool dense_o = may && R > 256, dense_down = may && R > 448;
   // The attention takes finished (rotated, bf16) q, k and v: the tcgen05 form, and the cache-fill forward, whose K/V go to
   // the cache.  (A function of the node width, never of the number of nodes.)

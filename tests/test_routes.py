@@ -43,3 +43,23 @@ def test_lm_head_takes_no_slower_kernel(rule):
     for (case, times), dense in zip(LM_HEAD.items(), took):
         assert within(times[dense], times[0]), (case, dense)
     assert within(sum(t[d] for t, d in zip(LM_HEAD.values(), took)), sum(min(t) for t in LM_HEAD.values()))
+
+
+# (gate|up features, d, rows): without, with the evenly shared kernel
+GATE_UP = {
+    (1408, 256, 192): (7.5, 5.3), (1408, 256, 256): (6.5, 5.4), (11264, 2048, 192): (15.4, 13.4), (24576, 4096, 192): (47.2, 39.3),
+    (28672, 4096, 192): (50.2, 46.5), (37888, 4096, 192): (57.2, 57.4), (37888, 4096, 256): (58.4, 60.8), (38912, 4096, 192): (88.1, 67.9),
+    (38912, 4096, 256): (81.2, 72.9), (45056, 4096, 192): (91.3, 73.5), (45056, 4096, 256): (80.1, 78.3), (49152, 4096, 192): (95.9, 80.2),
+    (49152, 2048, 192): (52.4, 42.4), (51200, 4096, 192): (100.7, 81.5), (53248, 4096, 192): (102.6, 88.2), (53248, 4096, 256): (85.6, 90.0),
+    (57344, 4096, 192): (105.9, 96.3), (57344, 4096, 256): (112.3, 100.8), (65536, 4096, 192): (112.2, 105.1), (65536, 4096, 256): (114.5, 109.1),
+    (67584, 4096, 176): (99.9, 104.2), (67584, 2048, 256): (53.8, 58.1), (75776, 4096, 192): (121.0, 120.5), (75776, 4096, 256): (117.4, 124.9),
+    (76800, 4096, 192): (154.7, 125.1), (76800, 4096, 256): (146.0, 133.9), (79872, 4096, 192): (151.8, 131.1), (90112, 2048, 192): (86.1, 73.3),
+    (90112, 2048, 256): (67.3, 74.4),
+}
+
+
+def test_gate_up_takes_no_slower_kernel(rule):
+    took = rule([f"gemm_wave_gains({n}, {int(r > 240)})" for n, _, r in GATE_UP])
+    for (case, times), even in zip(GATE_UP.items(), took):
+        assert within(times[even], times[0]), (case, even)
+    assert within(sum(t[e] for t, e in zip(GATE_UP.values(), took)), sum(min(t) for t in GATE_UP.values()))
