@@ -751,17 +751,7 @@ int launch_attention_verify_pipe(cudaStream_t st, const AttnArgs& a, int n_parts
   g.npt = qt_rows / T;
   if (g.npt > kKeys / g.t_pad) g.npt = kKeys / g.t_pad;
   const int q_tiles = (rps + g.npt * T - 1) / (g.npt * T);
-  // How many CTAs share the parts: one for each, one for two, or one for all - the bits are the same.  One CTA to an SM, so many
-  // query tiles take turns if each part has a CTA of its own.  A turn costs some 8 us and 1.5 us a tile, the exchange 3 us, merging
-  // in registers 0.6 us a part (in tenths below; fitted to 1, 2 and 4 CTAs at 5, 9 and 17 tiles).
-  g.n_ctas = g.n_parts;
-  long long best = 0;
-  for (int n : {g.n_parts, g.n_parts / 2, 1}) {
-    if (n < 1 || g.n_parts % n != 0) continue;
-    const long long turns = ((long long)a.H * a.n_seq_slots * q_tiles * n + kSms - 1) / kSms;
-    const long long cost = turns * (80 + 15 * ((g.n_all + n - 1) / n) + (n > 1 ? 30 : 0) + 6 * (g.n_parts / n - 1));
-    if (best == 0 || cost < best) { best = cost; g.n_ctas = n; }
-  }
+  g.n_ctas = attn_pipe_ctas(g.n_parts, g.n_all, (long long)a.H * a.n_seq_slots * q_tiles, qt_rows);      // (the bits are the same)
   const float scale_log2 = (1.0f / sqrtf((float)a.hd)) * 1.4426950408889634f;
   const size_t smem = (size_t)kTileBytes * (2 + kStagesK + kStagesV) + 16384 + 128 + 1024;   // Q, P, K and V stages, softmax exchange
   alignas(64) CUtensorMap tm[5];

@@ -2,6 +2,8 @@
 // about bits, so they may look at the rows of a forward.
 #pragma once
 
+#include <initializer_list>
+
 namespace ssd {
 
 // The rules that share work out take the machine's size from here; a grid of persistent CTAs asks the device.
@@ -54,6 +56,31 @@ inline bool gemm_wave_gains(int N, bool dense) {
   const int other = dense ? ceil_div(ceil_div(N, 256), kSms / 2) * 128 : tiles <= kSms ? 128 : ceil_div(tiles, 2 * kSms) * 256;
   const WaveShare share = wave_share(N, 1);
   return share.turns == 1 ? 4 * other >= 5 * share.couples : 8LL * other >= 9LL * share.turns * share.couples;
+}
+
+// CTAs that share the `parts` of the key tiles of each (query tile, head, sequence) in the tcgen05 attention, `work` of these in all: one
+// for each part, one for two, or one for all of them.  An SM has one CTA and a GPC room for few clusters, so clusters take
+// turns: in tenths of a us, a turn of CTAs with a part each costs 52 to 74 and 12 to 18 a tile (tiles of 32, 64 and 128 query rows),
+// one of CTAs with several 32 to 68, 12 to 21 a tile (128 rows: scores are read twice there) and 15 to 24 where they have something to
+// exchange.  Fitted to 730 sizes (4 to 60 heads, 2 to 33 tiles, 32 to 640 rows): 1 % above the best choice at the most in all but
+// 21, where the heads are 40 and more.  us a launch with one CTA, with half as many as parts and with as many:
+//   2 tiles in 2 parts, 128 rows      32 heads 14.3 / - / 11.1       5 tiles in 4 parts  32 heads, 32 rows 12.5 / 11.1 / 9.2
+//   17 tiles in 2 parts, 512 rows     40 heads 79.0 / - / 67.5       160 rows            20.0 / 18.7 / 23.7
+//   3 tiles in 3 parts, 256 rows      24 heads 17.3 / - / 21.3       17 in 8, 8 heads, 256 rows  43.2 / 23.1 / 28.0
+inline int attn_pipe_ctas(int parts, int tiles, long long work, int query_rows) {
+  constexpr int kClusters[9] = {0, kSms, kSms / 2, 45, 33, 24, 18, 15, 15};       // of as many CTAs that find an SM each
+  const int at = query_rows <= 32 ? 0 : query_rows <= 64 ? 1 : 2;
+  constexpr int kTurn[3] = {52, 59, 74}, kTile[3] = {12, 12, 18}, kTurnShared[3] = {32, 33, 68}, kTileShared[3] = {12, 14, 21}, kExchange[3] = {15, 22, 24};
+  int ctas = parts;
+  long long best = 0;
+  for (const int n : {parts, parts / 2, 1}) {
+    if (n < 1 || parts % n != 0) continue;
+    const long long turns = ceil_div(work, kClusters[n < 8 ? n : 8]), tiles_each = ceil_div(tiles, n);
+    const long long cost = n == parts ? 18 + turns * (kTurn[at] + kTile[at] * tiles_each)
+                                      : 30 + turns * (kTurnShared[at] + kTileShared[at] * tiles_each + (n > 1 ? kExchange[at] : 0));
+    if (best == 0 || cost < best) { best = cost; ctas = n; }
+  }
+  return ctas;
 }
 
 }  // namespace ssd

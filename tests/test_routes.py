@@ -63,3 +63,39 @@ def test_gate_up_takes_no_slower_kernel(rule):
     for (case, times), even in zip(GATE_UP.items(), took):
         assert within(times[even], times[0]), (case, even)
     assert within(sum(t[e] for t, e in zip(GATE_UP.values(), took)), sum(min(t) for t in GATE_UP.values()))
+
+
+# (parts, key tiles, query tiles x heads x sequences, rows of a query tile): by the CTAs that share the parts
+ATTENTION = {
+    (2, 2, 32, 128): {1: 13.2, 2: 10.1},
+    (2, 17, 160, 128): {1: 79.0, 2: 67.5},
+    (3, 3, 48, 128): {1: 17.3, 3: 21.3},
+    (4, 5, 32, 32): {1: 12.9, 2: 11.2, 4: 9.2},
+    (4, 5, 64, 128): {1: 19.3, 2: 18.4, 4: 22.9},
+    (8, 17, 16, 128): {1: 43.2, 4: 23.1, 8: 28.0},
+    (8, 9, 16, 32): {1: 18.3, 4: 11.8, 8: 17.0},
+    (8, 33, 16, 128): {1: 72.5, 4: 31.8, 8: 36.4},
+    (7, 7, 24, 128): {1: 26.9, 7: 22.9},
+    (2, 2, 4, 64): {1: 9.6, 2: 8.6},
+    (2, 3, 48, 128): {1: 14.9, 2: 11.9},
+    (2, 17, 180, 128): {1: 86.4, 2: 70.3},
+    (2, 2, 40, 128): {1: 13.7, 2: 9.9},
+    (4, 33, 160, 128): {1: 144.7, 2: 129.9, 4: 121.2},
+    (7, 7, 16, 128): {1: 25.2, 7: 20.7},
+    (4, 4, 160, 128): {1: 34.1, 2: 44.7, 4: 51.5},
+    (4, 4, 28, 128): {1: 18.1, 2: 16.4, 4: 12.1},
+    (8, 33, 16, 128): {1: 71.7, 4: 30.0, 8: 34.6},
+    (3, 3, 48, 64): {1: 11.5, 3: 16.9},
+}
+
+
+def test_attention_takes_no_slower_cluster(rule):
+    took = rule([f"attn_pipe_ctas({p}, {t}, {w}, {q})" for p, t, w, q in ATTENTION])
+    for (case, times), ctas in zip(ATTENTION.items(), took):
+        assert within(times[ctas], min(times.values())), (case, ctas)
+
+
+def test_attention_has_whole_clusters_of_its_parts(rule):
+    sizes = [(p, t, w, q) for p in range(2, 9) for t in (p, 2 * p + 1, 257) for w in (1, 33, 149, 4096) for q in (32, 64, 128)]
+    for (parts, *_), ctas in zip(sizes, rule(["attn_pipe_ctas(%d, %d, %d, %d)" % s for s in sizes])):
+        assert ctas in (1, parts, parts / 2)
