@@ -43,8 +43,6 @@ constexpr int kEpiPitch = 132;       // floats per row of the epilogue's transpo
 constexpr int kEpiBufFloats = 32 * kEpiPitch;     // a group's transpose buffer: one chunk
 constexpr unsigned long long kWaitLimitNs = 2000000000ull;   // default bound of a wait, 2 s: far beyond any legitimate one
 
-constexpr int kPairedResidualCtas = 112;         // CTAs in clusters of pairs that all find an SM (14 clusters of eight)
-
 struct TcParams {
   int R, N, K;
   int row_blocks;  // per weight tile
@@ -769,12 +767,9 @@ int launch_gemm_tc(cudaStream_t st, const GemmArgs& g) {
   p.w_tiled = g.w_tiled;
   // Pairs of tiles as one two-SM MMA from `two_sm_min_rows` padded rows on (0: never): every SM then takes
   // in half of the activation tile.  The accumulation order is the same, so the row count may decide.
-  // EPI_RESIDUAL: a cluster is then twice as large, and of eight CTAs with an SM each the GPCs have room for 15; so only where that
-  // is enough, or where there are row blocks to take turns anyway.  us in the live stream, without / with: 28 tiles in four
-  // splits, K 18944: 128 rows 30.3 / 29.0, 256 rows 46.0 / 39.8, 320 rows 54.5 / 47.8, 384 rows 72.8 / 58.5; 32 tiles, K 12288: 288
-  // rows 38.8 / 35.5, 384 rows 52.8 / 46.3, but 416 rows 57.2 / 60.3 and 128 rows (16 clusters, two turns) 24.7 / 43.1.
+  // EPI_RESIDUAL: a cluster is then twice as large.
   const bool pairs_fit = g.epi != EPI_RESIDUAL ||
-                         (2 * g.splits <= kGemmMaxClusterSplits && (gemm_tiles(g.N) * g.splits <= kPairedResidualCtas || (p.row_blocks > 1 && p.npad <= 192)));
+                         (2 * g.splits <= kGemmMaxClusterSplits && residual_pairs(gemm_tiles(g.N), g.splits, (g.K + kBlockK - 1) / kBlockK, p.row_blocks, p.npad));
   p.two_sm = (g.two_sm_min_rows > 0 && p.npad >= g.two_sm_min_rows && g.epi != EPI_SUM && pairs_fit && (gemm_tiles(g.N) % 2) == 0) ? 1 : 0;
   uint32_t cols = 32;
   while ((int)cols < p.npad) cols <<= 1;

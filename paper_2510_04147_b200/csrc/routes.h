@@ -83,4 +83,25 @@ inline int attn_pipe_ctas(int parts, int tiles, long long work, int query_rows) 
   return ctas;
 }
 
+// O and down in the skinny kernel as pairs of tiles, whose clusters are twice as large (2 * splits CTAs).  A pair pays from 8 K
+// blocks a split on (below, its set-up and the wider exchange outweigh half of the copies), and only where all clusters find
+// room at once: of eight CTAs with an SM each the GPCs take 14 or 15, of CTAs that share an SM (more CTAs than SMs) twice that.
+// 32 clusters of these still pay with long splits and blocks of up to 192 rows, the more the longer; with 416 rows they do not
+// (57.2 / 60.3).  us, single tiles / pairs (28 tiles: d 3584, and so on), four splits:
+//   K blocks each   128 rows       256 rows       288 rows       352 rows
+//   8 tiles   4     8.5 / 9.1      12.2 / 13.1    9.2 / 9.8      9.7 / 10.3
+//   20 tiles  8     9.9 / 9.9      14.6 / 15.0    15.9 / 15.5    19.7 / 16.7
+//   24 tiles 12     11.4 / 11.4    16.2 / 16.4    19.1 / 18.4    23.7 / 20.2
+//   24 tiles 32     17.8 / 17.3    24.8 / 24.0    27.3 / 24.9    34.8 / 27.6
+//   28 tiles 74     30.0 / 29.1    43.4 / 38.6    47.7 / 42.3    64.8 / 47.1
+//   16 tiles  4     8.2 / 8.9      12.4 / 13.0    10.2 / 20.1 (128 CTAs with an SM each: two turns)
+//   32 tiles        24.7 / 43.1 (K 12288: 16 clusters)   12 each 19.8 / 20.5; 24 24.8 / 36.6; 32 28.5 / 28.1, 352 rows 36.2 / 29.0;
+//                   48 36.0 / 33.2, 47.3 / 35.8; 56 39.7 / 40.3, 52.3 / 49.7; 64 44.1 / 46.9, 58.8 / 51.0; 74 49.4 / 44.9, 68.1 / 50.5
+inline bool residual_pairs(int tiles, int splits, int k_blocks, int row_blocks, int block_rows) {
+  const int ctas = tiles * splits * row_blocks, each = k_blocks / splits;
+  const bool share = ctas > kSms;
+  if (ctas <= (share ? 2 : 1) * 112) return each >= 8;
+  return share && row_blocks > 1 && block_rows <= 192 && each >= 32;
+}
+
 }  // namespace ssd
