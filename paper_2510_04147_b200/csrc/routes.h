@@ -61,16 +61,15 @@ inline bool gemm_wave_gains(int N, bool dense) {
 // CTAs that share the `parts` of the key tiles of each (query tile, head, sequence) in the tcgen05 attention, `work` of these in all: one
 // for each part, one for two, or one for all of them.  An SM has one CTA and a GPC room for few clusters, so clusters take
 // turns: in tenths of a us, a turn of CTAs with a part each costs 52 to 74 and 12 to 18 a tile (tiles of 32, 64 and 128 query rows),
-// one of CTAs with several 32 to 68, 12 to 21 a tile (128 rows: scores are read twice there) and 15 to 24 where they have something to
-// exchange.  Fitted to 730 sizes (4 to 60 heads, 2 to 33 tiles, 32 to 640 rows): 1 % above the best choice at the most in all but
-// 21, where the heads are 40 and more.  us a launch with one CTA, with half as many as parts and with as many:
+// one of CTAs with several 32 to 64, 12 to 20 a tile (128 rows: scores are read twice there) and 15 to 24 where they have something to
+// exchange.  Fitted to 730 sizes (4 to 60 heads, 2 to 33 tiles, 32 to 640 rows): the best choice within 3 % in all but 8.  us a launch with one CTA, with half as many as parts and with as many:
 //   2 tiles in 2 parts, 128 rows      32 heads 14.3 / - / 11.1       5 tiles in 4 parts  32 heads, 32 rows 12.5 / 11.1 / 9.2
 //   17 tiles in 2 parts, 512 rows     40 heads 79.0 / - / 67.5       160 rows            20.0 / 18.7 / 23.7
 //   3 tiles in 3 parts, 256 rows      24 heads 17.3 / - / 21.3       17 in 8, 8 heads, 256 rows  43.2 / 23.1 / 28.0
 inline int attn_pipe_ctas(int parts, int tiles, long long work, int query_rows) {
   constexpr int kClusters[9] = {0, kSms, kSms / 2, 45, 33, 24, 18, 15, 15};       // of as many CTAs that find an SM each
   const int at = query_rows <= 32 ? 0 : query_rows <= 64 ? 1 : 2;
-  constexpr int kTurn[3] = {52, 59, 74}, kTile[3] = {12, 12, 18}, kTurnShared[3] = {32, 33, 68}, kTileShared[3] = {12, 14, 21}, kExchange[3] = {15, 22, 24};
+  constexpr int kTurn[3] = {52, 59, 74}, kTile[3] = {12, 12, 18}, kTurnShared[3] = {32, 33, 64}, kTileShared[3] = {12, 14, 20}, kExchange[3] = {15, 22, 24};
   int ctas = parts;
   long long best = 0;
   for (const int n : {parts, parts / 2, 1}) {

@@ -86,6 +86,7 @@ ATTENTION = {
     (4, 4, 28, 128): {1: 18.1, 2: 16.4, 4: 12.1},
     (8, 33, 16, 128): {1: 71.7, 4: 30.0, 8: 34.6},
     (3, 3, 48, 64): {1: 11.5, 3: 16.9},
+    (5, 5, 32, 128): {1: 19.5, 5: 21.3},
 }
 
 
