@@ -329,8 +329,13 @@ gemm_dense_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant
   } else if (warp == 1) {
     // ------------------------------------------------------------------ MMA issuer (the even CTA, for both)
     // One lane, elected once, walks the whole loop: with warp-uniform addresses and descriptors an MMA is a few instructions
-    // (from a diverged lane's registers each took 70 clocks to issue, 580 per K block in all).
-    if (leader && elect_one()) {
+    // (from a diverged lane's registers each took 70 clocks to issue, 580 per K block in all).  Of 256-feature residual tiles, whose
+    // epilogue is the one that spills, the whole warp walks it and one lane issues: the compiler then spills less there (loads of
+    // 584 bytes for 608).  us of O and down, d 4096, one lane / the warp: 700 rows 33.1 / 32.0 and 73.7 / 70.9, 1024 rows 35.5 / 34.6
+    // and 76.7 / 73.9; of 128-feature tiles, 1536 rows, 43.7 / 48.1 and 111.9 / 125.4.
+    constexpr bool kWarpWalks = kFeat == 256 && kEpi == EPI_RESIDUAL;
+    auto all = [](bool v) -> bool { return kWarpWalks ? __all_sync(0xffffffffu, v) != 0 : v; };
+    if (leader && (kWarpWalks || elect_one())) {
       const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(kFeat >> 3) << 17) | ((uint32_t)(kTileRows >> 4) << 24);
       bool ok = true;
       const uint32_t full0 = smem_addr(full_bar), empty0 = smem_addr(empty_bar);
@@ -341,26 +346,30 @@ gemm_dense_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant
         for (int split = 0; split < p.splits && ok; ++split, ++nth) {
           const int buf = nth % kBufs;
           if (nth >= kBufs) {
-            ok = mbar_wait(smem_addr(&acc_empty[buf]), (uint32_t)((nth / kBufs) & 1) ^ 1u, abort_flag, p.wait_limit_ns);
+            ok = all(mbar_wait(smem_addr(&acc_empty[buf]), (uint32_t)((nth / kBufs) & 1) ^ 1u, abort_flag, p.wait_limit_ns));
             if (!ok) break;
             tc_fence_after();
           }
           const uint32_t tmem_d = tmem_base + (uint32_t)(buf * kFeat);
           const int kb0 = split * n_kb / p.splits, kb1 = (split + 1) * n_kb / p.splits;
           for (int kb = kb0; kb < kb1; ++kb) {
-            ok = mbar_wait(full0 + 8 * s, phase, abort_flag, p.wait_limit_ns);
+            ok = all(mbar_wait(full0 + 8 * s, phase, abort_flag, p.wait_limit_ns));
             if (!ok) break;
             // (the address field of a descriptor counts 16-byte units: a stage and a k16 step are additions)
             const uint64_t xd = xdesc0 + (uint32_t)(s * (kStageBytes >> 4)), wd = wdesc0 + (uint32_t)(s * (kStageBytes >> 4));
+            if (!kWarpWalks || elect_one()) {
 #pragma unroll
-            for (int k = 0; k < kBlockK / 16; ++k) tc_mma_bf16_pair(tmem_d, xd + 2 * k, wd + 2 * k, idesc, (uint32_t)(((kb - kb0) | k) != 0));
-            tc_commit_pair(empty0 + 8 * s);
+              for (int k = 0; k < kBlockK / 16; ++k) tc_mma_bf16_pair(tmem_d, xd + 2 * k, wd + 2 * k, idesc, (uint32_t)(((kb - kb0) | k) != 0));
+              tc_commit_pair(empty0 + 8 * s);
+              if (kWarpWalks && kb + 1 == kb1) tc_commit_pair(smem_addr(&acc_full[buf]));
+            }
+            if (kWarpWalks) __syncwarp();
             if (++s == kStages) { s = 0; phase ^= 1u; }
           }
-          if (ok) tc_commit_pair(smem_addr(&acc_full[buf]));
+          if (!kWarpWalks && ok) tc_commit_pair(smem_addr(&acc_full[buf]));
         }
       }
-      if (!ok) { *abort_flag = 1; raise_word(p.err_flag, 2); }
+      if (!ok && (!kWarpWalks || lane == 0)) { *abort_flag = 1; raise_word(p.err_flag, 2); }
     }
     __syncwarp();
   } else {
