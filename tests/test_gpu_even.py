@@ -1,6 +1,8 @@
 """The evenly shared projections (q|k|v and gate|up of up to 256 rows) against the skinny kernel: the same K ranges in the same
 order, so the bits of a forward are the same.  Row counts around the halves of a CTA pair (8-row steps, quarters of 32 rows, 128),
-units that end inside a weight tile, one and two MMAs to a unit, one and four K splits."""
+units that end inside a weight tile, one and two MMAs to a unit, one and four K splits, one to four units to a pair one after the
+other.  (With dense_rows = 0 every projection that fits takes this kernel, whether that is faster or not; test_routes.py has the
+units of these widths.)"""
 import numpy as np
 import pytest
 
@@ -15,6 +17,13 @@ SHAPES = {
     # four K splits with accumulators of their own; units of 136 and of 256 couples (two MMAs)
     "splits": BASE.replace(name="even_splits", d_model=1024, n_heads=28, n_kv_heads=4, d_ffn=9664),
     "wide": BASE.replace(name="even_wide", d_model=512, n_heads=32, n_kv_heads=32, d_ffn=18944),
+    # two units to a pair and one accumulator: of 136 couples over a single K block (each of the two producer warps has every
+    # second unit to itself), of 200 over three and of 256 over five, more than the ring has stages
+    "two_turns": BASE.replace(name="even_two_turns", n_layers=1, d_model=64, n_heads=2, n_kv_heads=1, d_ffn=19456),
+    "two_turns_3": BASE.replace(name="even_two_turns_3", n_layers=1, d_model=184, n_heads=2, n_kv_heads=1, d_ffn=28672),
+    "two_turns_5": BASE.replace(name="even_two_turns_5", n_layers=1, d_model=320, n_heads=2, n_kv_heads=1, d_ffn=37888),
+    # four units to a pair, the last ones missing
+    "four_turns": BASE.replace(name="even_four_turns", n_layers=1, d_model=128, n_heads=2, n_kv_heads=1, d_ffn=60008),
 }
 
 
@@ -22,6 +31,7 @@ SHAPES = {
     ("narrow", 5, 1, 1), ("narrow", 33, 13, 1), ("narrow", 250, 13, 13), ("narrow", 256, 24, 9),
     ("splits", 17, 16, 1), ("splits", 255, 23, 11), ("splits", 161, 32, 8),
     ("wide", 9, 9, 2), ("wide", 129, 24, 7), ("wide", 256, 16, 16),
+    ("two_turns", 7, 3, 1), ("two_turns", 161, 32, 8), ("two_turns_3", 200, 23, 11), ("two_turns_5", 256, 32, 5), ("four_turns", 33, 32, 7),
 ])
 def test_even_and_skinny_projections_give_the_same_bits(shape, prompt, block, nodes):
     from paper_2510_04147_b200 import binding
