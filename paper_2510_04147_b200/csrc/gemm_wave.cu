@@ -20,8 +20,9 @@
 // Bound by the weights (HBM) and, for narrow units, by the tensor pipe (256 rows whatever `half` is).  At 256 rows gate|up of d 4096,
 // ffn 12288 streams its 201 MB in 32 us of the kernel's 40; the rest is the ramp and the epilogue.  us in the live stream, before /
 // now: 256 rows q|k|v 39 / 32, gate|up 54 / 43; 216 rows 37 (with its finishing pass) / 29, 50 / 41; 128 rows 31 / 31, 41 / 43, so
-// fewer rows stay with gemm.cu, which leaves SMs to the kernel behind it.  Above 256 rows the units would take turns, and the
-// dense kernel's tiles have their epilogue under the next tile's main loop.  Every wait is bounded as in gemm.cu.
+// fewer rows stay with gemm.cu, which leaves SMs to the kernel behind it.  More than 256 rows, which a pair has no room for at once,
+// are the dense kernel's, whose tiles have their epilogue under the next tile's main loop.  Every wait is bounded as in gemm.cu, and
+// the tensor memory, all of it, is never waited for: an SM has registers for one of these CTAs and for no other that holds any.
 #include "kernels.h"
 
 #include <cuda.h>
@@ -49,8 +50,8 @@ constexpr unsigned long long kWaitLimitNs = 2000000000ull;
 struct WaveParams {
   int R, K, couples;     // couples: N / 2
   int splits;            // K ranges with an accumulator each
-  int half;              // rows of a CTA; a tile is 2 half rows
-  int m_tiles, units;
+  int half;              // rows of a CTA
+  int units;
   int cpu;               // couples of a unit
   int n0, n1;            // features of the two MMAs (n1 = 0: one)
   int stages, stage_bytes, bufs;
@@ -185,7 +186,7 @@ gemm_wave_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant_
   uint64_t* bars = reinterpret_cast<uint64_t*>(sTrans + kTransBytes<kEpi> + kListBytes);
   uint64_t* full_bar = bars;                       // leader: both CTAs' bytes of a stage
   uint64_t* empty_bar = bars + kMaxStages;         // each CTA: its stage may be refilled
-  uint64_t* acc_full = bars + 2 * kMaxStages;      // each CTA: a tile's accumulators are complete
+  uint64_t* acc_full = bars + 2 * kMaxStages;      // each CTA: a unit's accumulators are complete
   uint64_t* acc_empty = acc_full + kMaxBufs;       // leader: the epilogue warps of the pair have read them
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(acc_empty + kMaxBufs);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
@@ -197,7 +198,6 @@ gemm_wave_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant_
   const int crank = blockIdx.x & 1;         // rank in the cluster of two
   const bool leader = crank == 0;
   const int pair = blockIdx.x >> 1, n_pairs = gridDim.x >> 1;
-  const int total = p.m_tiles * p.units;
   const int acc_cols = p.n0 + p.n1;
 
   if (threadIdx.x == 0) {
@@ -244,9 +244,9 @@ gemm_wave_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant_
       const uint32_t smem0 = smem_addr(smem), full0 = smem_addr(full_bar);
       pdl_wait();
       int s = 0;
-      for (int tile = pair; tile < total && s < p.stages; tile += n_pairs)
+      for (int unit = pair; unit < p.units && s < p.stages; unit += n_pairs)
         for (int kb = 0; kb < n_kb && s < p.stages; ++kb, ++s)
-          tma_load_2d_pair(smem0 + s * p.stage_bytes, &tmX, full0 + 8 * s, kb * kBlockK, (2 * (tile % p.m_tiles) + crank) * p.half);
+          tma_load_2d_pair(smem0 + s * p.stage_bytes, &tmX, full0 + 8 * s, kb * kBlockK, crank * p.half);
     }
     __syncwarp();
   } else if (warp >= kEpiEnd) {
@@ -258,12 +258,12 @@ gemm_wave_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant_
       bool ok = true;
       const uint32_t smem0 = smem_addr(smem), full0 = smem_addr(full_bar), empty0 = smem_addr(empty_bar);
       int4* const box = s_box + turn * kMaxBoxes;
-      int n_box = 0, x_row = 0;
+      int n_box = 0;
+      const int x_row = crank * p.half;
       bool waited = false;
       uint32_t bytes = 0;                    // of a stage, both CTAs
-      auto enter = [&](int tile) {           // the copies of a unit: its couples cut at the weight tiles, and powers of two of them in one
-        const int unit = tile / p.m_tiles, c0 = unit * p.cpu, n = min(p.cpu, p.couples - c0);
-        x_row = (2 * (tile - unit * p.m_tiles) + crank) * p.half;
+      auto enter = [&](int unit) {           // the copies of a unit: its couples cut at the weight tiles, and powers of two of them in one
+        const int c0 = unit * p.cpu, n = min(p.cpu, p.couples - c0);
         bytes = 2u * (uint32_t)((p.half + n) * kBlockK * 2);
         n_box = 0;
         for (int done = 0; done < n;) {
@@ -274,13 +274,13 @@ gemm_wave_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant_
         }
       };
       enter(pair);
-      int tile = pair, s = turn, round = 0;
+      int unit = pair, s = turn, round = 0;
       for (int kb = turn;; s += kProducers, kb += kProducers) {
         while (s >= p.stages) { s -= p.stages; ++round; }
         if (kb >= n_kb) {
-          do { kb -= n_kb; tile += n_pairs; } while (kb >= n_kb);
-          if (tile >= total) break;
-          enter(tile);
+          do { kb -= n_kb; unit += n_pairs; } while (kb >= n_kb);
+          if (unit >= p.units) break;
+          enter(unit);
         }
         const uint32_t fb = full0 + 8 * s, dst = smem0 + s * p.stage_bytes;
         if (round > 0) {
@@ -316,7 +316,7 @@ gemm_wave_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant_
       const int stage_units = p.stage_bytes >> 4;      // (the address field of a descriptor counts 16-byte units)
       int s = 0, nth = 0;                    // stage; tiles so far
       uint32_t phase = 0;
-      for (int tile = pair; tile < total && ok; tile += n_pairs, ++nth) {
+      for (int unit = pair; unit < p.units && ok; unit += n_pairs, ++nth) {
         const int buf = nth % p.bufs;
         if (nth >= p.bufs) {
           ok = mbar_wait(smem_addr(&acc_empty[buf]), (uint32_t)((nth / p.bufs) & 1) ^ 1u, abort_flag, p.wait_limit_ns);
@@ -354,12 +354,11 @@ gemm_wave_kernel(const __grid_constant__ CUtensorMap tmX, const __grid_constant_
     bool ok = true;
     int nth = 0;
     uint8_t* trans = sTrans + (warp - 2) * kTransWarp<kEpi>;
-    for (int tile = pair; tile < total; tile += n_pairs, ++nth) {
-      const int unit = tile / p.m_tiles, mt = tile - unit * p.m_tiles;
+    for (int unit = pair; unit < p.units; unit += n_pairs, ++nth) {
       const int c0 = unit * p.cpu, n = min(p.cpu, p.couples - c0);
       // this warp's rows: [row0, row0 + 32) as far as the CTA's half goes
-      const int row0 = (2 * mt + crank) * p.half + quad * 32, row = row0 + lane;
-      const int row_end = min(p.R, (2 * mt + crank + 1) * p.half);
+      const int row0 = crank * p.half + quad * 32, row = row0 + lane;
+      const int row_end = min(p.R, (crank + 1) * p.half);
       const bool live = row < row_end, any = row0 < row_end;
       float inv = 1.f;
       if (live) {                            // RMSNorm, consumer side: the producers' per-tile sums in slot order
@@ -534,8 +533,7 @@ int launch(cudaStream_t st, const GemmArgs& g, WaveParams p, int dev) {
     attr_set[dev] = true;
   }
   const int smem = p.stages * p.stage_bytes + fixed + behind;
-  const int total = p.m_tiles * p.units, pairs = kSms / 2;
-  const dim3 grid(2 * (total < pairs ? total : pairs));
+  const dim3 grid(2 * (p.units < kSms / 2 ? p.units : kSms / 2));
   return launch_pdl_cluster(gemm_wave_kernel<kEpi, kWide>, grid, dim3(kThreads<kEpi>), (size_t)smem, st, 2u, tmX, tmW, p) == cudaSuccess ? 0 : -4;
 }
 
@@ -543,9 +541,7 @@ int unit_columns(int cpu) { return 2 * ((cpu + 15) & ~15); }
 
 }  // namespace
 
-bool gemm_wave_fits(int N, int R, int splits) {
-  return N % 128 == 0 && splits * unit_columns(wave_share(N, (R + 255) / 256).couples) <= 512;
-}
+bool gemm_wave_fits(int N, int R, int splits) { return N % 128 == 0 && R <= 256 && splits * unit_columns(wave_share(N).couples) <= 512; }
 
 int launch_gemm_wave(cudaStream_t st, const GemmArgs& g) {
   if ((g.x_pitch % 8) || (((uintptr_t)g.x) & 15) || (((uintptr_t)g.w) & 15) || !g.w_tiled || !g.sq || g.sq_count < 1 || g.norm_dim < 1) return -2;
@@ -553,11 +549,10 @@ int launch_gemm_wave(cudaStream_t st, const GemmArgs& g) {
   if (g.epi == EPI_QKV ? (!g.qkv || g.qkv->hd != 128) : (g.epi != EPI_SWIGLU || g.splits != 1 || !g.act)) return -2;
   WaveParams p{};
   p.R = g.R; p.K = g.K; p.couples = g.N / 2; p.splits = g.splits;
-  p.m_tiles = (g.R + 255) / 256;
-  p.half = ((g.R + 2 * p.m_tiles - 1) / (2 * p.m_tiles) + 7) & ~7;
+  p.half = ((g.R + 1) / 2 + 7) & ~7;
   const int dev = device_slot();
   if (dev < 0) return -4;
-  p.cpu = wave_share(g.N, p.m_tiles).couples;
+  p.cpu = wave_share(g.N).couples;
   p.units = (p.couples + p.cpu - 1) / p.cpu;
   const int cols = unit_columns(p.cpu);
   p.n0 = p.cpu < 128 ? cols : 256;

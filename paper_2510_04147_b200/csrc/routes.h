@@ -33,11 +33,11 @@ inline bool lm_head_dense(int V, int K, int R) {
 // Evenly shared projections (gemm_wave.cu): the couples of a feature and its partner that make a unit, in as few turns as the width of an
 // accumulator allows, one unit for every pair of SMs in each.
 struct WaveShare { int turns, couples; };
-inline WaveShare wave_share(int N, int m_tiles) {
-  const long long work = (long long)(N / 2) * m_tiles, pairs = kSms / 2;
+inline WaveShare wave_share(int N) {
+  const int pairs = kSms / 2;
   for (int turns = 1;; ++turns) {
-    const long long couples = (ceil_div(work, pairs * turns) + 7) & ~7;
-    if (couples <= 256) return {turns, couples < 16 ? 16 : (int)couples};
+    const int couples = (ceil_div(N / 2, (long long)pairs * turns) + 7) & ~7;
+    if (couples <= 256) return {turns, couples < 16 ? 16 : couples};
   }
 }
 
@@ -54,7 +54,7 @@ inline WaveShare wave_share(int N, int m_tiles) {
 inline bool gemm_wave_gains(int N, bool dense) {
   const int tiles = ceil_div(N, 128);
   const int other = dense ? ceil_div(ceil_div(N, 256), kSms / 2) * 128 : tiles <= kSms ? 128 : ceil_div(tiles, 2 * kSms) * 256;
-  const WaveShare share = wave_share(N, 1);
+  const WaveShare share = wave_share(N);
   return share.turns == 1 ? 4 * other >= 5 * share.couples : 8LL * other >= 9LL * share.turns * share.couples;
 }
 

@@ -67,7 +67,7 @@ def test_gate_up_takes_no_slower_kernel(rule):
 
 def test_units_of_the_widths_that_test_gpu_even_takes(rule):
     pads = (256, 9664, 18944, 19456, 28672, 37888, 60032)          # gates, in whole weight tiles
-    got = rule([f"wave_share(2 * {f}, 1).{what}" for f in pads for what in ("turns", "couples")])
+    got = rule([f"wave_share(2 * {f}).{what}" for f in pads for what in ("turns", "couples")])
     assert list(zip(got[::2], got[1::2])) == [(1, 16), (1, 136), (1, 256), (2, 136), (2, 200), (2, 256), (4, 208)]
 
 
