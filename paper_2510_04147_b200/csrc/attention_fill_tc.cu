@@ -21,7 +21,8 @@
 // Per pair of query tiles and key tile 3500 clocks were measured (clock64) where 2048 are the bound: a warpgroup takes 210 to
 // read its scores, 240 for the maximum, 1370 for exponentials and P, then waited 1280 for PV and the next S behind it, and the
 // MMA warp was idle for 720.  Issuing PV in two halves takes half of it out of that wait, and registers shifted from the
-// warps that need few to the softmax threads take out their spills: 512 tokens 16.7 -> 15.0 us alone, dream's 1024 43.5 ->
+// warps that need few to the softmax threads take out nearly all of their spills (12 bytes of stores are left with one query tile, 48
+// with two): 512 tokens 16.7 -> 15.0 us alone, dream's 1024 43.5 ->
 // 39.3, eight times 509 73 -> 71.  4096 tokens (880 TFLOP/s at full clocks) run under the power cap, 290 to 330 us before and
 // 270 to 310 now, and took 1900 in the mma.sync form with its merge pass.  Taking 2 to 4 of 8 exponentials to the FMA pipe (a
 // polynomial on packed pairs) gave nothing more.

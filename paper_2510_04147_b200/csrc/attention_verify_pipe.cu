@@ -25,21 +25,21 @@
 // owner merges in part order.  With several query tiles a CTA of its own for every part is more CTAs than SMs, in two or three
 // turns: then each CTA has two parts, or all of them, one after the other, and merges them in registers - the same parts and the
 // same operations, so the same bits.  us a layer (live stream), a CTA for every part / now: 512 keys, 32 heads, 160 rows 27.8 /
-// 21.6, 320 rows 45.2 / 28.6; 1024 keys, 28 heads, 192 rows 32.2 / 25.7, 320 rows 51.6 / 36.6; two sequences of 700 keys, 28 heads,
-// 64 rows 17.8 / 11.6.
+// 21.3, 320 rows 45.2 / 27.2; 1024 keys, 28 heads, 192 rows 32.2 / 23.9, 320 rows 51.6 / 33.4; two sequences of 700 keys, 28 heads,
+// 64 rows 17.8 / 11.4.
 //
 // Bound by the serial chain of a tile, not by bytes, except for long prefixes under small query tiles.  Of a 128-row tile's
 // 3400 clocks (clock64 at each step, 4096 keys) the scores' maximum took 580, the wait for O += P V 425, exponentials, sums and P
-// 1850, of which the special-function unit accounts for 1024.  Taken out: the visibility test of every key (masked scores become
-// -inf where they are loaded) and that wait: 4 sequences of 4096 keys 77 -> 72 us at 128 rows each, 1536 keys 24.2 -> 22.9.
-// Four threads to a row, or even and odd tiles in two streams, were no faster.  A thread keeps its scores in registers from the maximum
-// to the exponentials, 64 of them under 128 rows, where the outputs of parts in one CTA do not need those registers (kShared; with
-// them spilled, 28 heads at 320 rows 35 -> 49 us): read twice / kept, us a layer: 4 sequences of 4096 keys, 128 rows each 88 / 79; 8 of 509 keys, 96
-// rows each 50.5 / 42.1; one sequence, 512 keys, 128 rows 17.3 / 14.7; 1024 keys, 28 heads, 128 rows 17.9 / 15.6.
-// us per layer in the live stream (the forms before it, which summed and rotated the projection's split-K partials themselves, in
-// brackets; finishing q, k and v is now a pass of 3 to 10 us): one sequence, 512 keys, 32 / 64 / 128 rows 10 (15) / 13 (20) /
-// 19 (32); 1536 keys, 128 rows 23 (43); 8 sequences of 512 keys 27 (38); 4 of 4096 keys, 64 / 128 rows each 56 (83) / 72
-// (108); 3 sequences of 777 keys with nodes of 24 rows, which only the mma.sync form took, 25 (160).
+// 1850, of which the special-function unit accounts for 1024.  The visibility test of every key (masked scores become -inf where
+// they are loaded) and that wait are out of it.  Four threads to a row, or even and odd tiles in two streams, were no faster.  A
+// thread keeps its scores in registers from the maximum to the exponentials, 64 of them under 128 rows; where the outputs of
+// several parts in one CTA need those registers (kShared) it reads them twice, with 52 bytes of spills (with the scores kept
+// as well, 28 heads at 320 rows 35 -> 49 us).  Read twice / kept, us a layer: 8 sequences of 509 keys, 96 rows each 50.5 / 42.1;
+// one of 512 keys, 128 rows 17.3 / 14.7; 1024 keys, 28 heads, 128 rows 17.9 / 15.6.
+// us a layer in the live stream, 32 heads (in brackets forms that summed and rotated the projection's split-K partials
+// themselves; finishing q, k and v is a pass of 3 to 7 us below 161 rows and part of the projection from there on): one
+// sequence, 512 keys, 32 / 64 / 128 rows 8.6 (15) / 10.3 (20) / 14.5 (32); 1536 keys, 128 rows 19.1 (43); 8 sequences of 512 keys,
+// 32 rows each 25.0 (38); 4 of 4096 keys, 64 / 128 rows each 54.5 (83) / 78.9 (108); 3 sequences of 777 keys with nodes of 24 rows, which only the mma.sync form took, 25.0 (160).
 #include "attn_common.cuh"
 
 #include <cuda.h>

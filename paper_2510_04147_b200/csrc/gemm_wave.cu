@@ -18,7 +18,8 @@
 // whatever the stage held before; they only reach accumulator rows and columns that nothing reads.
 //
 // Bound by the weights (HBM) and, for narrow units, by the tensor pipe (256 rows whatever `half` is).  At 256 rows gate|up of d 4096,
-// ffn 12288 streams its 201 MB in 32 us of the kernel's 40; the rest is the ramp and the epilogue.  us in the live stream, before /
+// ffn 12288 streams its 201 MB in 32 us of the kernel's 41; the rest is the ramp and the epilogue (alone and cold, 44 us, either limit is
+// reached for 57 % of the launch, q|k|v's 32 us for 40 %).  us in the live stream, before /
 // now: 256 rows q|k|v 39 / 32, gate|up 54 / 43; 216 rows 37 (with its finishing pass) / 29, 50 / 41; 128 rows 31 / 31, 41 / 43, so
 // fewer rows stay with gemm.cu, which leaves SMs to the kernel behind it.  More than 256 rows, which a pair has no room for at once,
 // are the dense kernel's, whose tiles have their epilogue under the next tile's main loop.  Every wait is bounded as in gemm.cu, and

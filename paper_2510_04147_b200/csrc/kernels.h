@@ -303,7 +303,7 @@ int gemm_tiles(int N);
 // summed in order: the bits of the skinny kernel (and launch_qkv_finish) with the same splits.  Returns 0 or a negative
 // ssd error code.
 int launch_gemm_dense(cudaStream_t st, const GemmArgs& g);
-// A few hundred rows: the features shared out evenly over all SMs, tile-contiguous weights; EPI_QKV (head dimension 128) or
+// Up to 256 rows: the features shared out evenly over all SMs, tile-contiguous weights; EPI_QKV (head dimension 128) or
 // EPI_SWIGLU.  The same sums as the other kernels with the same splits.  Returns 0 or a negative ssd error code.
 int launch_gemm_wave(cudaStream_t st, const GemmArgs& g);
 bool gemm_wave_fits(int N, int R, int splits);     // its accumulators have room for the K splits

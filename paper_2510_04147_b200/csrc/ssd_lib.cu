@@ -194,7 +194,8 @@ int capped_split(int s, int k) {
 // A power of two: clusters of five leave so many SMs of a GPC unused that 140 CTAs take two waves (28 tiles: 1019 -> 1164 us).
 // Up to four splits may be down to one K block: the cluster of the splits shares the rows of the epilogue, which is most of a small
 // launch.  (d 256, ffn 688: one split of O's four K blocks and two of down's eleven took 91 us a forward of 16 to 80 rows, four
-// of each 86, four and eight 87.)
+// of each 86, four and eight 87.  The dense kernel, which has to add up the same splits, pays for it: O of 257 and more rows 7.8 -> 8.9
+// us, a prefill of 700 and more tokens 1 % slower.)
 int auto_split_residual(int tiles, int k) {
   const int kb = (k + 63) / 64;
   int s = 8;
@@ -438,7 +439,9 @@ int forward(ssd_ctx* c, int kind, const int* ids_dev, int R, RowMap map, int n_s
   // Of 161 to 256 rows, q|k|v and gate|up share their features out evenly (where that is less than the turns of whole tiles).  us of
   // eight layers with the LM head, neither / q|k|v / gate|up, d 4096, ffn 12288 (96 and 192 tiles): 128 rows 1241 / 1251 / 1262,
   // 160 1420 / 1410 / 1422, 192 1545 / 1533 / 1499, 224 1742 / 1692 / 1660, 256 1766 / 1696 / 1705; d 3584, ffn 18944 (36 tiles of
-  // four splits; 296 tiles go evenly as they are): 128 rows 1307 / 1300 / 1343, 192 1596 / 1575 / 1613, 256 1773 / 1738 / 1783.
+  // four splits; 296 tiles go evenly as they are): 128 rows 1307 / 1300 / 1343, 192 1596 / 1575 / 1613, 256 1773 / 1738 / 1783.  q|k|v of
+  // 192 rows in other widths, skinny with its finishing pass / even: d 1024 23 / 22, d 2048 26 / 24, d 3072 30 / 29, d 5120 38 / 39 (256
+  // rows 42 / 40).
   const bool two_thirds = 3LL * R > 2LL * c->dense_rows;      // (the option may be any int: a very large one means never)
   const bool anywhere = c->dense_rows == 0;                   // (0: wherever these kernels can run, not only where they are the faster ones)
   const bool even = R <= 256 && two_thirds;
