@@ -769,7 +769,7 @@ int launch_gemm_tc(cudaStream_t st, const GemmArgs& g) {
   // in half of the activation tile.  The accumulation order is the same, so the row count may decide.
   // EPI_RESIDUAL: a cluster is then twice as large.
   const bool pairs_fit = g.epi != EPI_RESIDUAL ||
-                         (2 * g.splits <= kGemmMaxClusterSplits && residual_pairs(gemm_tiles(g.N), g.splits, (g.K + kBlockK - 1) / kBlockK, p.row_blocks, p.npad));
+                         (2 * g.splits <= kGemmMaxClusterSplits && residual_pairs(gemm_tiles(g.N), g.splits, (g.K + kBlockK - 1) / kBlockK, p.row_blocks, p.npad, g.before));
   p.two_sm = (g.two_sm_min_rows > 0 && p.npad >= g.two_sm_min_rows && g.epi != EPI_SUM && pairs_fit && (gemm_tiles(g.N) % 2) == 0) ? 1 : 0;
   uint32_t cols = 32;
   while ((int)cols < p.npad) cols <<= 1;

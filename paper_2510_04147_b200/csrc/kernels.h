@@ -291,6 +291,7 @@ struct GemmArgs {
   int sq_count, sq_stride, norm_dim;
   float norm_eps;
   // EPI_RESIDUAL: splits = cluster size (<= kGemmMaxClusterSplits)
+  int before;            // CTAs of the kernel in front where that is the skinny one with two to an SM, else 0
   const QkvOut* qkv;     // EPI_QKV (host pointer, copied into the launch)
   float* h;              // [R][N] fp32 residual stream, updated in place
   bf16* hb;              // [R][N] bf16(h * gain)

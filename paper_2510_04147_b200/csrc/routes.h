@@ -86,7 +86,9 @@ inline int attn_pipe_ctas(int parts, int tiles, long long work, int query_rows) 
 // blocks a split on (below, its set-up and the wider exchange outweigh half of the copies), and only where all clusters find
 // room at once: of eight CTAs with an SM each the GPCs take 14 or 15, of CTAs that share an SM (more CTAs than SMs) twice that.
 // 32 clusters of these still pay with long splits and blocks of up to 192 rows, the more the longer; with 416 rows they do not
-// (57.2 / 60.3).  us, single tiles / pairs (28 tiles: d 3584, and so on), four splits:
+// (57.2 / 60.3), and not where the kernel in front, which is of the same kind (`before` CTAs, two to an SM), fills half of the
+// machine in its last turn: one place in every SM is free then, clusters are spread over those, and the last of them have to
+// wait.  (Where it leaves most places free, or none, the clusters lie close.)  us, single tiles / pairs (28 tiles: d 3584, and so on), four splits:
 //   K blocks each   128 rows       256 rows       288 rows       352 rows
 //   8 tiles   4     8.5 / 9.1      12.2 / 13.1    9.2 / 9.8      9.7 / 10.3
 //   20 tiles  8     9.9 / 9.9      14.6 / 15.0    15.9 / 15.5    19.7 / 16.7
@@ -95,12 +97,14 @@ inline int attn_pipe_ctas(int parts, int tiles, long long work, int query_rows) 
 //   28 tiles 74     30.0 / 29.1    43.4 / 38.6    47.7 / 42.3    64.8 / 47.1
 //   16 tiles  4     8.2 / 8.9      12.4 / 13.0    10.2 / 20.1 (128 CTAs with an SM each: two turns)
 //   32 tiles        24.7 / 43.1 (K 12288: 16 clusters)   12 each 19.8 / 20.5; 24 24.8 / 36.6; 32 28.5 / 28.1, 352 rows 36.2 / 29.0;
-//                   48 36.0 / 33.2, 47.3 / 35.8; 56 39.7 / 40.3, 52.3 / 49.7; 64 44.1 / 46.9, 58.8 / 51.0; 74 49.4 / 44.9, 68.1 / 50.5
-inline bool residual_pairs(int tiles, int splits, int k_blocks, int row_blocks, int block_rows) {
+//                   48 36.0 / 33.2, 47.3 / 35.8; 74 49.4 / 44.9, 68.1 / 50.5.  Last turn 51 % full: 56 39.8 / 44, 384 rows 55 / 72;
+//                   59 % (K 24576) 61 / 85, 88 / 105; 62 % (K 15360) 43 / 52, 57 / 71; 38 % (K 22528) 58 / 52, 82 / 71; 84 % (K 17408) 47 / 43, 65 / 54
+inline bool residual_pairs(int tiles, int splits, int k_blocks, int row_blocks, int block_rows, int before) {
   const int ctas = tiles * splits * row_blocks, each = k_blocks / splits;
   const bool share = ctas > kSms;
   if (ctas <= (share ? 2 : 1) * 112) return each >= 8;
-  return share && row_blocks > 1 && block_rows <= 192 && each >= 32;
+  const int last_turn = before % (2 * kSms) * 100 / (2 * kSms);        // per cent of the places
+  return share && row_blocks > 1 && block_rows <= 192 && each >= 32 && (last_turn < 45 || last_turn >= 75);
 }
 
 }  // namespace ssd

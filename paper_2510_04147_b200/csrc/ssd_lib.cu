@@ -570,6 +570,7 @@ int forward(ssd_ctx* c, int kind, const int* ids_dev, int R, RowMap map, int n_s
     g.splits = c->split_down; g.epi = EPI_PARTIAL; g.out = c->partial;
     const float* gain = (l + 1 < c->cfg.n_layers) ? c->L[l + 1].g_attn : c->g_final;
     produce_norm(g, gain, c->split_down);
+    if (!even_gu && !dense_gu) g.before = gemm_tiles(2 * c->ffn_pad) * ceil_div(R, 256);
     rc = dense_down ? run_gemm_dense(c, g, SSD_PROF_GEMM_DOWN) : run_gemm(c, g, SSD_PROF_GEMM, SSD_PROF_GEMM_DOWN);
     if (rc) return rc;
   }
