@@ -30,7 +30,7 @@ METRIC = "decode tokens/s at batch 1 (LLaDA-8B-shaped) and % HBM roofline per ve
 # DRAM bytes per projection launch from the ncu capture summarised in
 # profiles/projections_and_attention_llada8b_4layers_counters.md (mean over the four projections of a LLaDA-8B-shaped layer).
 # Valid only for the kernel source it was taken from: reported as null once gemm.cu has changed.
-GEMM_TRAFFIC = {"workload": "llada8b", "bytes_per_launch": 113.1e6, "gemm_cu_sha256_16": "c6e81e7cfb4a8452"}
+GEMM_TRAFFIC = {"workload": "llada8b", "bytes_per_launch": 112.8e6, "gemm_cu_sha256_16": "bb80a9668ba21021"}
 FALLBACK_PEAKS = {"hbm_gbs": 6650.0, "bf16_tflops": 1590.0, "bf16_tflops_sustained": 1400.0}
 
 
